@@ -327,9 +327,8 @@ __device__ __forceinline__ void merge_levels(KeyT* bufX, KeyT* bufY, const int* 
       const int d0 = blk * kBlockItems;
       const int m = (L - d0) < kBlockItems ? (L - d0) : kBlockItems;
       if (lenA != 0 && lenB != 0) {
-        const int a0 = warp_corank(A, lenA, B, lenB, d0, lane);
-        const int a1 =
-            (d0 + m == L) ? lenA : warp_corank(A, lenA, B, lenB, d0 + m, lane, a0, a0 + m);
+        int a0, a1;
+        block_coranks(A, lenA, B, lenB, d0, m, lane, a0, a1);
         const int X = a1 - a0;
         if (m <= kSmallBlockMax)
           warp_merge_small<KeyT>(A + a0, X, B + (d0 - a0), m - X, dst + outo + d0, lane,

@@ -81,13 +81,17 @@ __device__ __forceinline__ void cas(KeyT& a, KeyT& b) {
   b = hi;
 }
 // 64-bit keys: one unsigned 64-bit compare drives the four 32-bit selects of
-// the pair (min and max computed apart would each compare and select).
+// the pair.  In PTX, because written as conditional expressions it is compiled
+// as a min and a max that compare once each (four compare instructions a
+// pair instead of two; a fifth of the 8-byte tile sort's instructions).
 __device__ __forceinline__ void cas(uint64_t& a, uint64_t& b) {
-  const bool sw = b < a;
-  const uint64_t lo = sw ? b : a;
-  const uint64_t hi = sw ? a : b;
-  a = lo;
-  b = hi;
+  asm("{\n\t.reg .pred p;\n\t.reg .b32 al, ah, bl, bh, xl, xh, yl, yh;\n\t"
+      "setp.lt.u64 p, %1, %0;\n\t"
+      "mov.b64 {al, ah}, %0;\n\tmov.b64 {bl, bh}, %1;\n\t"
+      "selp.b32 xl, bl, al, p;\n\tselp.b32 xh, bh, ah, p;\n\t"
+      "selp.b32 yl, al, bl, p;\n\tselp.b32 yh, ah, bh, p;\n\t"
+      "mov.b64 %0, {xl, xh};\n\tmov.b64 %1, {yl, yh};\n\t}\n"
+      : "+l"(a), "+l"(b));
 }
 
 // Compare-exchange whose direction is chosen per lane: with flip set the
@@ -102,12 +106,15 @@ __device__ __forceinline__ void cas_dir(KeyT& a, KeyT& b, bool flip) {
 }
 // 64-bit keys: the direction folds into the compare's predicate (swap when
 // the pair is out of the lane's order), then four 32-bit selects.
-__device__ __forceinline__ void cas_dir(uint64_t& a, uint64_t& b, bool flip) {
-  const bool sw = (b < a) != flip;
-  const uint64_t x = sw ? b : a;
-  const uint64_t y = sw ? a : b;
-  a = x;
-  b = y;
+__device__ __forceinline__ void cas_dir(uint64_t& a, uint64_t& b, uint32_t f) {
+  asm("{\n\t.reg .pred p, q;\n\t.reg .b32 al, ah, bl, bh, xl, xh, yl, yh;\n\t"
+      "setp.ne.u32 q, %2, 0;\n\tsetp.lt.xor.u64 p, %1, %0, q;\n\t"
+      "mov.b64 {al, ah}, %0;\n\tmov.b64 {bl, bh}, %1;\n\t"
+      "selp.b32 xl, bl, al, p;\n\tselp.b32 xh, bh, ah, p;\n\t"
+      "selp.b32 yl, al, bl, p;\n\tselp.b32 yh, ah, bh, p;\n\t"
+      "mov.b64 %0, {xl, xh};\n\tmov.b64 %1, {yl, yh};\n\t}\n"
+      : "+l"(a), "+l"(b)
+      : "r"(f));
 }
 
 // ---------------------------------------------------------------------------
@@ -180,17 +187,21 @@ __device__ __forceinline__ void cas_mix(uint32_t& a, uint32_t& b, int i,
   }
 }
 
-// 64-bit pair: swap when sw, the selects as multiply-adds (exact for f in
-// {0, 1}).
+// 64-bit pair, swapped when out of the order f asks for (0: ascending): the
+// lower key's halves are selected, the other key's halves are what is left of the
+// two sums (x in {a, b}, so a + b - x is the other one, exact modulo 2^32).
 template <typename M>
-__device__ __forceinline__ void swap64_mad(uint64_t& a, uint64_t& b, bool sw, const M& c) {
-  const uint32_t f = sw ? c.one : 0u;
-  const uint32_t al = (uint32_t)a, ah = (uint32_t)(a >> 32);
-  const uint32_t bl = (uint32_t)b, bh = (uint32_t)(b >> 32);
-  const uint32_t dl = mad_u32(al, c.m1, bl), el = mad_u32(bl, c.m1, al);   // bl - al, al - bl
-  const uint32_t dh = mad_u32(ah, c.m1, bh), eh = mad_u32(bh, c.m1, ah);
-  const uint32_t xl = mad_u32(f, dl, al), yl = mad_u32(f, el, bl);         // sw ? b : a, sw ? a : b
-  const uint32_t xh = mad_u32(f, dh, ah), yh = mad_u32(f, eh, bh);
+__device__ __forceinline__ void cas64_mad(uint64_t& a, uint64_t& b, uint32_t f, const M& c) {
+  const uint32_t sl = mad_u32((uint32_t)a, c.one, (uint32_t)b);
+  const uint32_t sh = mad_u32((uint32_t)(a >> 32), c.one, (uint32_t)(b >> 32));
+  uint32_t xl, xh;
+  asm("{\n\t.reg .pred p, q;\n\t.reg .b32 al, ah, bl, bh;\n\t"
+      "setp.ne.u32 q, %4, 0;\n\tsetp.lt.xor.u64 p, %3, %2, q;\n\t"
+      "mov.b64 {al, ah}, %2;\n\tmov.b64 {bl, bh}, %3;\n\t"
+      "selp.b32 %0, bl, al, p;\n\tselp.b32 %1, bh, ah, p;\n\t}\n"
+      : "=r"(xl), "=r"(xh)
+      : "l"(a), "l"(b), "r"(f));
+  const uint32_t yl = mad_u32(xl, c.m1, sl), yh = mad_u32(xh, c.m1, sh);
   a = ((uint64_t)xh << 32) | xl;
   b = ((uint64_t)yh << 32) | yl;
 }
@@ -199,7 +210,7 @@ template <int MIX, int MIXD, int MIX64, int MIXD64>
 __device__ __forceinline__ void cas_mix(uint64_t& a, uint64_t& b, int i,
                                         const Mix<MIX, MIXD, MIX64, MIXD64>& c) {
   if (mad_pick(i, MIX64))
-    swap64_mad(a, b, b < a, c);
+    cas64_mad(a, b, 0u, c);
   else
     cas(a, b);
 }
@@ -223,9 +234,9 @@ template <int MIX, int MIXD, int MIX64, int MIXD64>
 __device__ __forceinline__ void cas_dir_mix(uint64_t& a, uint64_t& b, uint32_t f, int i,
                                             const Mix<MIX, MIXD, MIX64, MIXD64>& c) {
   if (mad_pick(i, MIXD64))
-    swap64_mad(a, b, (b < a) != (f != 0), c);
+    cas64_mad(a, b, f, c);
   else
-    cas_dir(a, b, f != 0);
+    cas_dir(a, b, f);
 }
 
 // The mixes the kernels use (multiply-add pairs of 16: plain and per-lane
@@ -256,6 +267,16 @@ __device__ __forceinline__ void lds_if_lt(uint64_t& v, const uint64_t* p, int id
       : "+l"(v)
       : "r"(smem_u32addr(p)), "r"(idx), "r"(lim)
       : "memory");
+}
+__device__ __forceinline__ uint32_t lds_key(const uint32_t* p) {
+  uint32_t v;
+  asm volatile("ld.shared.b32 %0, [%1];" : "=r"(v) : "r"(smem_u32addr(p)) : "memory");
+  return v;
+}
+__device__ __forceinline__ uint64_t lds_key(const uint64_t* p) {
+  uint64_t v;
+  asm volatile("ld.shared.b64 %0, [%1];" : "=l"(v) : "r"(smem_u32addr(p)) : "memory");
+  return v;
 }
 // v = a[0] when idx < lim (signed), b[0] otherwise: one compare, two predicated
 // loads with complementary predicates (each touching consecutive words only).
@@ -299,14 +320,11 @@ __device__ __forceinline__ void lds_if_ge(uint64_t& v, const uint64_t* p, int id
 // ties taken from A (stable).  32-ary: each round all lanes probe positions
 // at an odd stride (distinct banks), a ballot narrows the range 32-fold.
 // ---------------------------------------------------------------------------
-// `lo0` / `hi0` narrow the search when a bracket is known: the co-rank of
-// d + m lies within [co-rank of d, co-rank of d + m] of the block before it.
 template <typename KeyT>
 __device__ __forceinline__ int warp_corank(const KeyT* A, int lenA, const KeyT* B, int lenB,
-                                           int d, int lane, int lo0 = 0, int hi0 = 0x7fffffff) {
-  int lo = d - lenB > lo0 ? d - lenB : lo0;
+                                           int d, int lane) {
+  int lo = d - lenB > 0 ? d - lenB : 0;
   int hi = d < lenA ? d : lenA;
-  hi = hi < hi0 ? hi : hi0;
   while (hi > lo) {
     const int step = ((hi - lo + 31) >> 5) | 1;
     const int i = lo + lane * step;
@@ -320,6 +338,46 @@ __device__ __forceinline__ int warp_corank(const KeyT* A, int lenA, const KeyT* 
     lo = nlo;
   }
   return lo;
+}
+
+// Both co-ranks of a full block, of d and of d + m, in one search: lanes 0-15
+// look for the first, lanes 16-31 for the second, each 16 probes a round (an odd
+// stride: at most two probes per bank).  Up to 4912 items in three rounds; one after
+// the other, 32 probes each, took five dependent rounds (the second search
+// bracketed by the first).
+template <typename KeyT>
+__device__ __forceinline__ void warp_corank_pair(const KeyT* A, int lenA, const KeyT* B, int lenB,
+                                                 int d, int m, int lane, int& c0, int& c1) {
+  const int dd = d + (lane < 16 ? 0 : m), l = lane & 15;
+  int lo = dd - lenB > 0 ? dd - lenB : 0;
+  int hi = dd < lenA ? dd : lenA;
+  while (__any_sync(0xffffffffu, hi > lo)) {
+    const int step = ((hi - lo + 15) >> 4) | 1;
+    const int i = lo + l * step;
+    bool p = true;                                 // positions >= hi count as "true"
+    if (i < hi) p = A[i] > B[dd - 1 - i];
+    const unsigned bal = __ballot_sync(0xffffffffu, p);
+    const unsigned hb = lane < 16 ? bal & 0xffffu : bal >> 16;
+    const int f = __ffs(hb) - 1;                   // first "true" probe, -1 if none
+    const int top = lo + f * step;
+    const int nlo = (f <= 0) ? (f == 0 ? lo : lo + 15 * step + 1) : top - step + 1;
+    hi = (f < 0) ? hi : (top < hi ? top : hi);
+    lo = nlo;
+  }
+  c0 = __shfl_sync(0xffffffffu, lo, 0);
+  c1 = __shfl_sync(0xffffffffu, lo, 16);
+}
+
+// Co-ranks a0 and a1 of the start and the end of a node's output block [d0, d0 + m).
+template <typename KeyT>
+__device__ __forceinline__ void block_coranks(const KeyT* A, int lenA, const KeyT* B, int lenB,
+                                              int d0, int m, int lane, int& a0, int& a1) {
+  if (d0 + m == lenA + lenB) {                       // the node's last block: its end is known
+    a0 = d0 == 0 ? 0 : warp_corank(A, lenA, B, lenB, d0, lane);
+    a1 = lenA;
+  } else {
+    warp_corank_pair(A, lenA, B, lenB, d0, m, lane, a0, a1);
+  }
 }
 
 // ---------------------------------------------------------------------------
@@ -340,9 +398,11 @@ __device__ __forceinline__ int warp_corank(const KeyT* A, int lenA, const KeyT* 
 // ---------------------------------------------------------------------------
 
 // Register k of lane l receives C[32k + l]: A[32k + l] when that is below X,
-// B[1023 - 32k - l] when it is at or above 1024 - Y, a pad in between.  The A
-// and B halves of a register are fetched by two predicated loads, so each
-// load instruction touches consecutive words only.
+// B[1023 - 32k - l] when it is at or above 1024 - Y, a pad in between.  Rows are
+// taken eight at a time: a group that lies in A or in B alone (three of four
+// of a full block) is eight plain loads; the others fetch the A and the B part
+// of a row by two predicated loads, so that each load instruction touches
+// consecutive words only.
 template <typename KeyT>
 __device__ __forceinline__ void warp_load_bitonic(const KeyT* A, int X, const KeyT* B, int Y,
                                                   KeyT (&v)[32], int lane) {
@@ -350,17 +410,46 @@ __device__ __forceinline__ void warp_load_bitonic(const KeyT* A, int X, const Ke
   const KeyT* pb = B + (kBlockItems - 1 - lane);     // C[32k+lane] = B[1023-32k-lane]
   const int xa = X - lane;                           // 32k + lane < X  <=>  32k < xa
   const int xb = kBlockItems - Y - lane;             // 32k + lane >= 1024 - Y  <=>  32k >= xb
-  if (X + Y == kBlockItems) {                        // full block: no pads, xa == xb
 #pragma unroll
-    for (int k = 0; k < 32; ++k) lds_pair(v[k], pa + 32 * k, pb - 32 * k, 32 * k, xa);
-    return;
+  for (int q = 0; q < 4; ++q) {
+    if (256 * (q + 1) <= X) {
+#pragma unroll
+      for (int k = 8 * q; k < 8 * q + 8; ++k) v[k] = lds_key(pa + 32 * k);
+    } else if (256 * q >= kBlockItems - Y) {
+#pragma unroll
+      for (int k = 8 * q; k < 8 * q + 8; ++k) v[k] = lds_key(pb - 32 * k);
+    } else {
+#pragma unroll
+      for (int k = 8 * q; k < 8 * q + 8; ++k) {
+        KeyT t = key_pad<KeyT>();
+        lds_if_lt(t, pa + 32 * k, 32 * k, xa);
+        lds_if_ge(t, pb - 32 * k, 32 * k, xb);
+        v[k] = t;
+      }
+    }
   }
+}
+
+// The same for a full block (X + Y = 1024): a row that is not in A or in B
+// alone takes one compare and two complementary predicated loads.
+template <typename KeyT>
+__device__ __forceinline__ void warp_load_bitonic_full(const KeyT* A, int X, const KeyT* B,
+                                                       KeyT (&v)[32], int lane) {
+  const KeyT* pa = A + lane;
+  const KeyT* pb = B + (kBlockItems - 1 - lane);
+  const int xa = X - lane;
 #pragma unroll
-  for (int k = 0; k < 32; ++k) {
-    KeyT t = key_pad<KeyT>();
-    lds_if_lt(t, pa + 32 * k, 32 * k, xa);
-    lds_if_ge(t, pb - 32 * k, 32 * k, xb);
-    v[k] = t;
+  for (int q = 0; q < 4; ++q) {
+    if (256 * (q + 1) <= X) {
+#pragma unroll
+      for (int k = 8 * q; k < 8 * q + 8; ++k) v[k] = lds_key(pa + 32 * k);
+    } else if (256 * q >= X) {
+#pragma unroll
+      for (int k = 8 * q; k < 8 * q + 8; ++k) v[k] = lds_key(pb - 32 * k);
+    } else {
+#pragma unroll
+      for (int k = 8 * q; k < 8 * q + 8; ++k) lds_pair(v[k], pa + 32 * k, pb - 32 * k, 32 * k, xa);
+    }
   }
 }
 
@@ -376,39 +465,99 @@ __device__ __forceinline__ int flip_mask(int lane) {
 // striped layout register k of lane l holds item 32k + l (row k, column l); in
 // the blocked layout lane l holds row l, item 32l + j in register j.
 
-// Half-cleaners of register distance D, D/2, .., 1 (strides 32D .. 32 of the
-// striped layout), ascending.
-template <int D, typename KeyT, typename M>
-__device__ __forceinline__ void striped_stages(KeyT (&v)[32], const M& c) {
-#pragma unroll
-  for (int s = D; s >= 1; s >>= 1) {
-#pragma unroll
-    for (int k = 0; k < 32; ++k)
-      if ((k & s) == 0) cas_mix(v[k], v[k + s], pair_ordinal(k, s), c);
-  }
-}
-
-// Striped -> blocked through `out` (16-byte aligned, 32 * nr items): row k is
-// stored with its 16-byte chunks XOR-swizzled by k & 7 (item 32k + l at word
-// 32k + (l ^ E*(k & 7))), so the scalar row stores and the 16-byte row loads
-// are both conflict-free.  Rows at or above nr are not stored; lanes at or
-// above nr receive pads.
-template <typename KeyT>
-__device__ __forceinline__ void striped_to_blocked(KeyT (&v)[32], KeyT* out, int nr, int lane) {
-  using V = Vec16<KeyT>;
-  constexpr int E = V::E;
+// Half-cleaner of register distance S (stride 32 S of the striped layout), ascending.
+template <int S, typename KeyT, typename M>
+__device__ __forceinline__ void striped_stage(KeyT (&v)[32], const M& c) {
 #pragma unroll
   for (int k = 0; k < 32; ++k)
-    if (k < nr) out[32 * k + (lane ^ (E * (k & 7)))] = v[k];
-  __syncwarp();
-  if (lane < nr) {
-    const typename V::T* row = reinterpret_cast<const typename V::T*>(out + 32 * lane);
-    const int sw = lane & 7;
+    if ((k & S) == 0) cas_mix(v[k], v[k + S], pair_ordinal(k, S), c);
+}
+
+// Transposes between the layouts go through shared memory.  stmatrix writes
+// four rows of 32 words with one instruction: lane T gives the address of
+// the 16 bytes that lanes 4 (T & 7) .. 4 (T & 7) + 3 hold of the row T >> 3.
+__device__ __forceinline__ void stsm_x4(uint32_t addr, uint32_t a, uint32_t b, uint32_t c,
+                                        uint32_t d) {
+  asm volatile("stmatrix.sync.aligned.m8n8.x4.shared.b16 [%0], {%1, %2, %3, %4};" ::"r"(addr),
+               "r"(a), "r"(b), "r"(c), "r"(d)
+               : "memory");
+}
+__device__ __forceinline__ uint4 lds128(uint32_t addr) {
+  uint4 x;
+  asm volatile("ld.shared.v4.b32 {%0, %1, %2, %3}, [%4];"
+               : "=r"(x.x), "=r"(x.y), "=r"(x.z), "=r"(x.w)
+               : "r"(addr)
+               : "memory");
+  return x;
+}
+__device__ __forceinline__ void sts32(uint32_t addr, uint32_t v) {
+  asm volatile("st.shared.b32 [%0], %1;" ::"r"(addr), "r"(v) : "memory");
+}
+
+// Rows 4q .. 4q + 3 of the striped layout to addr (+ 128: the high halves of 8-byte keys).
+__device__ __forceinline__ void store_rows4(uint32_t addr, const uint32_t* v) {
+  stsm_x4(addr, v[0], v[1], v[2], v[3]);
+}
+__device__ __forceinline__ void store_rows4(uint32_t addr, const uint64_t* v) {
+  stsm_x4(addr, (uint32_t)v[0], (uint32_t)v[1], (uint32_t)v[2], (uint32_t)v[3]);
+  stsm_x4(addr + 128, (uint32_t)(v[0] >> 32), (uint32_t)(v[1] >> 32), (uint32_t)(v[2] >> 32),
+          (uint32_t)(v[3] >> 32));
+}
+__device__ __forceinline__ void store_word(uint32_t addr, uint32_t v) { sts32(addr, v); }
+__device__ __forceinline__ void store_word(uint32_t addr, uint64_t v) {
+  sts32(addr, (uint32_t)v);
+  sts32(addr + 128, (uint32_t)(v >> 32));
+}
+// Keys 4 ch .. 4 ch + 3 of a row from the chunk at addr (+ 128 as above).
+__device__ __forceinline__ void load_chunk(uint32_t addr, uint32_t* v) {
+  const uint4 x = lds128(addr);
+  v[0] = x.x; v[1] = x.y; v[2] = x.z; v[3] = x.w;
+}
+__device__ __forceinline__ void load_chunk(uint32_t addr, uint64_t* v) {
+  const uint4 x = lds128(addr), y = lds128(addr + 128);
+  v[0] = ((uint64_t)y.x << 32) | x.x; v[1] = ((uint64_t)y.y << 32) | x.y;
+  v[2] = ((uint64_t)y.z << 32) | x.z; v[3] = ((uint64_t)y.w << 32) | x.w;
+}
+
+// Striped -> blocked through `out` (16-byte aligned, 32 * nr items).  Row k
+// takes the k-th 128 bytes (8-byte keys: 128 bytes of low halves, then 128 of
+// high halves) with its eight 16-byte chunks XOR-swizzled by k & 7, so the row
+// stores (stmatrix; a last group of fewer than four rows word by word) and
+// the 16-byte row loads are both conflict-free.  Rows at or above nr are not
+// stored; lanes at or above nr receive pads.
+template <typename KeyT>
+__device__ __forceinline__ void striped_to_blocked(KeyT (&v)[32], KeyT* out, int nr, int lane) {
+  constexpr uint32_t RB = 32 * sizeof(KeyT);
+  const uint32_t ob = smem_u32addr(out);
+  const uint32_t i = (uint32_t)lane >> 3, r = (uint32_t)lane & 7;
+  const uint32_t a0 = ob + i * RB + ((r ^ i) << 4);           // rows 8p + i
+  const uint32_t a1 = ob + i * RB + ((r ^ i ^ 4) << 4);       // rows 8p + 4 + i
+  const uint32_t row = ob + (uint32_t)lane * RB;
+  if (nr == 32) {
 #pragma unroll
-    for (int ch = 0; ch < 32 / E; ++ch) V::unpack(row[ch ^ sw], &v[ch * E]);
+    for (int q = 0; q < 8; ++q) store_rows4(((q & 1) ? a1 : a0) + 4 * q * RB, &v[4 * q]);
+    __syncwarp();
+#pragma unroll
+    for (int ch = 0; ch < 8; ++ch) load_chunk(row + ((ch ^ r) << 4), &v[4 * ch]);
   } else {
 #pragma unroll
-    for (int k = 0; k < 32; ++k) v[k] = key_pad<KeyT>();
+    for (int q = 0; q < 8; ++q) {
+      if (4 * q + 3 < nr) {
+        store_rows4(((q & 1) ? a1 : a0) + 4 * q * RB, &v[4 * q]);
+      } else {
+#pragma unroll
+        for (int k = 4 * q; k < 4 * q + 4; ++k)
+          if (k < nr) store_word(ob + k * RB + (((uint32_t)lane ^ (4 * (k & 7))) << 2), v[k]);
+      }
+    }
+    __syncwarp();
+    if (lane < nr) {
+#pragma unroll
+      for (int ch = 0; ch < 8; ++ch) load_chunk(row + ((ch ^ r) << 4), &v[4 * ch]);
+    } else {
+#pragma unroll
+      for (int k = 0; k < 32; ++k) v[k] = key_pad<KeyT>();
+    }
   }
   __syncwarp();
 }
@@ -447,7 +596,11 @@ __device__ __forceinline__ void blocked_stages(KeyT (&v)[32], int lane, const M&
 template <typename M, typename KeyT>
 __device__ __forceinline__ void warp_bitonic_1024(KeyT (&v)[32], KeyT* out, int nr, int lane) {
   const M c = mad_ones<M>();
-  striped_stages<16>(v, c);                          // strides 512 .. 32
+  striped_stage<16>(v, c);                           // strides 512 .. 32
+  striped_stage<8>(v, c);
+  striped_stage<4>(v, c);
+  striped_stage<2>(v, c);
+  striped_stage<1>(v, c);
   striped_to_blocked(v, out, nr, lane);
   blocked_stages<true>(v, lane, c);                  // strides 16 .. 1, store layout
 }
@@ -464,6 +617,28 @@ __device__ __forceinline__ void sts128(uint32_t addr, const uint32_t* v) {
 }
 __device__ __forceinline__ void sts128(uint32_t addr, const uint64_t* v) {
   asm volatile("st.shared.v2.b64 [%0], {%1, %2};" ::"r"(addr), "l"(v[0]), "l"(v[1]) : "memory");
+}
+
+template <typename KeyT>
+__device__ __forceinline__ KeyT lds_at(uint32_t addr) {
+  if constexpr (sizeof(KeyT) == 4) {
+    uint32_t v;
+    asm volatile("ld.shared.b32 %0, [%1];" : "=r"(v) : "r"(addr) : "memory");
+    return v;
+  } else {
+    uint64_t v;
+    asm volatile("ld.shared.b64 %0, [%1];" : "=l"(v) : "r"(addr) : "memory");
+    return v;
+  }
+}
+__device__ __forceinline__ void lds_chunk(uint32_t addr, uint32_t* v) {
+  asm volatile("ld.shared.v4.b32 {%0, %1, %2, %3}, [%4];"
+               : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3])
+               : "r"(addr)
+               : "memory");
+}
+__device__ __forceinline__ void lds_chunk(uint32_t addr, uint64_t* v) {
+  asm volatile("ld.shared.v2.b64 {%0, %1}, [%2];" : "=l"(v[0]), "=l"(v[1]) : "r"(addr) : "memory");
 }
 
 // 16-byte store when a <= b (signed), compare and store in one predicate.
@@ -613,12 +788,11 @@ __device__ __forceinline__ void warp_merge_any(const KeyT* A, int X, const KeyT*
 }
 
 // ---------------------------------------------------------------------------
-// One CTA merge level with a barrier after it (used by the base case, whose
-// blocks are all full).  Sequence q (q < 32) of `src` is described by lane
-// q's (off, len); sequences (2p, 2p+1) are merged into `dst`, pair outputs
-// packed in pair order, 16-byte aligned.  Work items are the 1024-item output
-// blocks of every pair, dealt to the warps round-robin.  next_seq() gives the
-// descriptors of the outputs.
+// One CTA merge level (used by the cluster base case).  Sequence q (q < 32)
+// of `src` is described by lane q's (off, len); sequences (2p, 2p+1) are merged
+// into `dst`, pair outputs packed in pair order, 16-byte aligned.  Work items
+// are the 1024-item output blocks of every pair, dealt to the warps
+// round-robin.
 // ---------------------------------------------------------------------------
 template <typename KeyT, typename M>
 __device__ __forceinline__ void cta_merge_level(const KeyT* src, KeyT* dst, int my_off, int my_len,
@@ -638,32 +812,13 @@ __device__ __forceinline__ void cta_merge_level(const KeyT* src, KeyT* dst, int 
     for (int d0 = 0; d0 < L; d0 += kBlockItems, ++item) {
       if (item % nwarps != warp) continue;
       const int m = (L - d0) < kBlockItems ? (L - d0) : kBlockItems;
-      const int a0 = warp_corank(A, a_len, B, b_len, d0, lane);
-      const int a1 = (d0 + m == L) ? a_len : warp_corank(A, a_len, B, b_len, d0 + m, lane, a0, a0 + m);
+      int a0, a1;
+      block_coranks(A, a_len, B, b_len, d0, m, lane, a0, a1);
       const int X = a1 - a0;
       warp_merge_block<KeyT, M>(A + a0, X, B + (d0 - a0), m - X, dst + outoff + d0, lane, xout);
     }
     outoff += (L + E - 1) / E * E;
   }
-}
-
-// Descriptors of the pair outputs of a level: lane p gets (packed offset, length).
-template <typename KeyT>
-__device__ __forceinline__ void next_seq(int& my_off, int& my_len, int nseq, int lane) {
-  constexpr int E = Vec16<KeyT>::E;
-  const int l0 = __shfl_sync(0xffffffffu, my_len, (2 * lane) & 31);
-  const int l1 = __shfl_sync(0xffffffffu, my_len, (2 * lane + 1) & 31);
-  int len = 0;
-  if (2 * lane < nseq) len = l0 + ((2 * lane + 1 < nseq) ? l1 : 0);
-  const int span = (len + E - 1) / E * E;
-  int incl = span;
-#pragma unroll
-  for (int o = 1; o < 32; o <<= 1) {
-    const int t = __shfl_up_sync(0xffffffffu, incl, o);
-    if (lane >= o) incl += t;
-  }
-  my_off = incl - span;
-  my_len = len;
 }
 
 // ---------------------------------------------------------------------------

@@ -16,10 +16,10 @@ constexpr int kMaxFanout = 32;
 // Compare-exchange pairs (of every 16 in a network stage) computed as one
 // min and two multiply-adds instead of min and max, per kernel: the base
 // case and the merge pass (plain pairs, pairs with a per-lane direction).
-constexpr int kTileMadPairs = 6, kTileMadDirPairs = 12;
+constexpr int kTileMadPairs = 8, kTileMadDirPairs = 12;
 constexpr int kMergeMadPairs = 0, kMergeMadDirPairs = 12;
 // The same for 64-bit keys (their selects as multiply-adds; see mms_common.cuh).
-constexpr int kTileMad64Pairs = 0, kTileMad64DirPairs = 0;
+constexpr int kTileMad64Pairs = 16, kTileMad64DirPairs = 0;
 constexpr int kMergeMad64Pairs = 6, kMergeMad64DirPairs = 0;
 
 // Device error word values (the first word of a sort workspace).
@@ -33,6 +33,15 @@ constexpr int kDevErrInternal = 2;      // a consistency check failed
 template <typename KeyT, int WARPS>
 struct MinBlocks {
   static constexpr int value = 3;
+};
+
+// CTAs per SM the base case is compiled for: 24 warps of 4-byte keys (80
+// registers), 16 warps of 8-byte keys (128 registers).  Its tile is sorted in one
+// buffer, so shared memory would take more; 32 warps of 4-byte keys (64
+// registers) measured the same, 20 of 8-byte keys (96) 5% slower.
+template <typename KeyT, int WARPS>
+struct TileMinBlocks {
+  static constexpr int value = (sizeof(KeyT) == 8 ? 16 : 24) / WARPS;
 };
 
 // CTAs per SM the partition variant of the merge pass is compiled for: two

@@ -192,7 +192,7 @@ __global__ void seg_desc_kernel(const unsigned long long* __restrict__ off, long
 // ---- persistent phase kernels ----------------------------------------------
 
 template <typename KeyT, int WARPS, bool XIN>
-__global__ void __launch_bounds__(WARPS * 32, (MinBlocks<KeyT, WARPS>::value))
+__global__ void __launch_bounds__(WARPS * 32, (TileMinBlocks<KeyT, WARPS>::value))
     seg_tile_sort_kernel(const KeyT* __restrict__ keys_in, KeyT* bufA, KeyT* bufB,
                          const Desc* __restrict__ desc, const int* __restrict__ total,
                          long long per_phase) {
@@ -209,7 +209,7 @@ __global__ void __launch_bounds__(WARPS * 32, (MinBlocks<KeyT, WARPS>::value))
 }
 
 template <int WARPS, bool XIN>
-__global__ void __launch_bounds__(WARPS * 32, (MinBlocks<uint64_t, WARPS>::value))
+__global__ void __launch_bounds__(WARPS * 32, (TileMinBlocks<uint64_t, WARPS>::value))
     seg_tile_sort_composite_kernel(const uint32_t* __restrict__ keys_in, uint64_t* bufA,
                                    uint64_t* bufB, const Desc* __restrict__ desc,
                                    const int* __restrict__ total, long long per_phase) {

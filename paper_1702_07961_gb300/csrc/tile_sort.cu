@@ -5,7 +5,7 @@
 namespace mms {
 
 template <typename KeyT, int WARPS, bool XIN, bool XOUT>
-__global__ void __launch_bounds__(WARPS * 32, (MinBlocks<KeyT, WARPS>::value))
+__global__ void __launch_bounds__(WARPS * 32, (TileMinBlocks<KeyT, WARPS>::value))
     tile_sort_kernel(const KeyT* __restrict__ in, KeyT* out, long long n) {
   extern __shared__ __align__(1024) unsigned char smem_raw[];
   constexpr int T = WARPS * kBlockItems;
@@ -16,7 +16,7 @@ __global__ void __launch_bounds__(WARPS * 32, (MinBlocks<KeyT, WARPS>::value))
 // Base case of the key-value sort: 32-bit keys -> sorted tiles of unique
 // 64-bit composites (ordered key << 32 | position in the array).
 template <int WARPS, bool XIN>
-__global__ void __launch_bounds__(WARPS * 32, (MinBlocks<uint64_t, WARPS>::value))
+__global__ void __launch_bounds__(WARPS * 32, (TileMinBlocks<uint64_t, WARPS>::value))
     tile_sort_composite_kernel(const uint32_t* __restrict__ in, uint64_t* out, long long n) {
   extern __shared__ __align__(1024) unsigned char smem_raw[];
   constexpr int T = WARPS * kBlockItems;
@@ -25,7 +25,7 @@ __global__ void __launch_bounds__(WARPS * 32, (MinBlocks<uint64_t, WARPS>::value
 }
 
 size_t tile_sort_smem_bytes(int key_bytes, int warps) {
-  return (size_t)key_bytes * 2 * (warps * kBlockItems + kTileSlack);
+  return (size_t)key_bytes * warps * kBlockItems;
 }
 
 template <typename KeyT, int WARPS, bool XIN, bool XOUT>
@@ -43,11 +43,13 @@ static cudaError_t launch_tile_sort_t(const void* in, void* out, long long n, cu
 template <int WARPS>
 static cudaError_t launch_tile_sort_w(int key_bytes, bool xin, bool xout, const void* in, void* out,
                                       long long n, cudaStream_t s) {
-  if (key_bytes == 8 && WARPS == 8) return cudaErrorInvalidValue;
-  if (key_bytes == 4) {
-    if (xin && xout) return launch_tile_sort_t<uint32_t, WARPS, true, true>(in, out, n, s);
-    if (xin) return launch_tile_sort_t<uint32_t, WARPS, true, false>(in, out, n, s);
-    return launch_tile_sort_t<uint32_t, WARPS, false, false>(in, out, n, s);
+  if (!valid_tile_warps(key_bytes, WARPS)) return cudaErrorInvalidValue;
+  if constexpr (WARPS != 2) {
+    if (key_bytes == 4) {
+      if (xin && xout) return launch_tile_sort_t<uint32_t, WARPS, true, true>(in, out, n, s);
+      if (xin) return launch_tile_sort_t<uint32_t, WARPS, true, false>(in, out, n, s);
+      return launch_tile_sort_t<uint32_t, WARPS, false, false>(in, out, n, s);
+    }
   }
   if constexpr (WARPS != 8) return launch_tile_sort_t<uint64_t, WARPS, false, false>(in, out, n, s);
   return cudaErrorInvalidValue;

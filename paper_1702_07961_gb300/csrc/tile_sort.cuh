@@ -8,10 +8,11 @@
 // with an in-register sorting network, the warp finishes its 1024 keys with
 // bitonic merges through conflict-free transposes in its share of the tile
 // buffer (the row/column transposes of shearsort, swizzled), and the CTA
-// merges the warps' blocks with the same conflict-free block merge the merge
-// rounds use.  HBM traffic: one coalesced 128-bit read and one coalesced
+// merges the warps' blocks with the same conflict-free networks, in place.  HBM traffic: one coalesced 128-bit read and one coalesced
 // 128-bit write of every key.
 #pragma once
+
+#include <type_traits>
 
 #include "mms_common.cuh"
 #include "mms_kernels.cuh"
@@ -48,65 +49,66 @@ __device__ __forceinline__ void lane_sort32(KeyT (&v)[32], const M& c) {
   }
 }
 
-// Blocked -> striped through `scratch` (16-byte aligned, 1024 items), with the
-// second half of every block of R rows read backwards.  On return register k
-// of lane l holds item 32k + l of the sequence in which every block of R rows
-// is its first R/2 rows in order followed by its last R/2 rows in reverse
-// (row qR + R - 1 - i into register qR + R/2 + i, column 31 - l into lane l):
-// a bitonic sequence when both halves of the block are ascending, so an
-// ascending half-cleaner cascade sorts it, with no per-lane directions.  Each
-// lane writes its row as 16-byte chunks XOR-swizzled by row & 7, and each
-// register load reads 32 distinct words of one row: no bank conflicts.
-template <int R, typename KeyT>
-__device__ __forceinline__ void blocked_to_striped_rev(KeyT (&v)[32], KeyT* scratch, int lane) {
+// Blocked -> striped through `scratch` (aligned to a row, 1024 items), with the
+// second half of every block of 2h rows read backwards (h a power of two, 1 ..
+// 16).  On return register k of lane l holds item 32k + l of the sequence in
+// which every block is its first h rows in order followed by its last h rows in
+// reverse, each from column 31 down: a bitonic sequence when both halves are
+// ascending, so an ascending half-cleaner cascade sorts it, with no per-lane
+// directions.  A lane of a second half writes its row to the mirrored place
+// (row l ^ (h - 1)), as 16-byte chunks XOR-swizzled by that place & 7; register k
+// is then column l, or 31 - l, of row k.  The writes and the reads (32 distinct words of one row) have no
+// bank conflicts.
+template <typename KeyT>
+__device__ __forceinline__ void blocked_to_striped_rev(KeyT (&v)[32], KeyT* scratch, int h,
+                                                       int lane) {
   constexpr int E = Vec16<KeyT>::E;
-  const uint32_t row = smem_u32addr(scratch + 32 * lane);
-  const int sw = lane & 7;
+  constexpr uint32_t SZ = sizeof(KeyT), RB = 32 * SZ;
+  const uint32_t sb = smem_u32addr(scratch);
+  const uint32_t place = (lane & h) ? lane ^ (h - 1) : lane;
+  const uint32_t row = (sb + place * RB) ^ ((place & 7) << 4);
 #pragma unroll
-  for (int ch = 0; ch < 32 / E; ++ch)
-    sts128(row + (uint32_t)((ch ^ sw) * E * (int)sizeof(KeyT)), &v[ch * E]);
+  for (int ch = 0; ch < 32 / E; ++ch) sts128(row ^ (ch << 4), &v[ch * E]);
+  __syncwarp();
+  // Column offsets: c[k] = lane, mirrored when k has bit h, swizzled by k & 7;
+  // c[k] follows from c[k without its lowest bit] by one XOR.
+  uint32_t mir[5];
+#pragma unroll
+  for (int b = 0; b < 5; ++b) mir[b] = (h >> b) & 1 ? 31 * SZ : 0u;
+  uint32_t c[32];
+  c[0] = sb ^ (lane * SZ);
+#pragma unroll
+  for (int k = 1; k < 32; ++k) {
+    const int p = k & (k - 1);                                 // k without its lowest bit
+    const int b = (k & -k) == 1 ? 0 : (k & -k) == 2 ? 1 : (k & -k) == 4 ? 2 : (k & -k) == 8 ? 3 : 4;
+    c[k] = c[p] ^ mir[b] ^ (uint32_t)(E * ((k & 7) ^ (p & 7)) * SZ);
+  }
+#pragma unroll
+  for (int k = 0; k < 32; ++k) v[k] = lds_at<KeyT>(c[k] + k * RB);
+  __syncwarp();
+}
+
+// Blocked layout -> `out` (aligned to a row, 1024 items) in order: the rows
+// go out swizzled, come back as consecutive 16-byte chunks (chunk 32q + lane in
+// registers), and those are stored in their places; all conflict-free.
+template <typename KeyT>
+__device__ __forceinline__ void blocked_to_linear(KeyT (&v)[32], KeyT* out, int lane) {
+  constexpr int E = Vec16<KeyT>::E;
+  constexpr int CPR = 32 / E;                                  // chunks of a row: 8 or 16
+  constexpr uint32_t RB = 32 * sizeof(KeyT);
+  const uint32_t sb = smem_u32addr(out);
+  const uint32_t row = (sb + lane * RB) ^ ((lane & 7) << 4);
+#pragma unroll
+  for (int ch = 0; ch < CPR; ++ch) sts128(row ^ (ch << 4), &v[ch * E]);
   __syncwarp();
 #pragma unroll
-  for (int k = 0; k < 32; ++k) {
-    const int kq = k % R;
-    const bool rev = kq >= R / 2;
-    const int src = rev ? k - kq + R - 1 - (kq - R / 2) : k;   // source row
-    const int w = rev ? 31 - lane : lane;                      // source column
-    v[k] = scratch[32 * src + (w ^ (E * (src & 7)))];
+  for (int q = 0; q < CPR; ++q) {
+    const uint32_t r = (uint32_t)(q * (32 / CPR)) + (uint32_t)lane / CPR;   // row of chunk 32q + lane
+    lds_chunk(sb + r * RB + ((((uint32_t)lane % CPR) ^ (r & 7)) << 4), &v[q * E]);
   }
   __syncwarp();
-}
-
-// One level of the warp sort: every block of R rows, whose two halves are
-// each sorted, becomes sorted (blocked layout in and out).
-template <int R, typename KeyT, typename M>
-__device__ __forceinline__ void warp_merge_rows(KeyT (&v)[32], KeyT* scratch, int lane,
-                                                const M& c) {
-  blocked_to_striped_rev<R>(v, scratch, lane);
-  striped_stages<R / 2>(v, c);                       // strides 16R .. 32
-  striped_to_blocked(v, scratch, 32, lane);
-  blocked_stages<false>(v, lane, c);                 // strides 16 .. 1
-}
-
-// Sorts 1024 keys held as 32 per lane (any assignment): each lane sorts its
-// 32 keys (a row), then levels of 64, 128, 256, 512 and 1024 keys merge pairs
-// of sorted blocks with bitonic cascades -- strides of 32 and more between
-// registers in the striped layout, the rest inside the lane -- through
-// conflict-free transposes in the warp's 1024-item `scratch` (no shuffles).
-// After the call register j of lane l holds sorted item 32*l + (j ^
-// flip_mask(l)), the layout warp_store_block writes out.
-template <typename KeyT>
-__device__ __forceinline__ void warp_sort_1024(KeyT (&v)[32], KeyT* scratch, int lane) {
-  const TileMix c = mad_ones<TileMix>();
-  lane_sort32(v, c);
-  warp_merge_rows<2>(v, scratch, lane, c);
-  warp_merge_rows<4>(v, scratch, lane, c);
-  warp_merge_rows<8>(v, scratch, lane, c);
-  warp_merge_rows<16>(v, scratch, lane, c);
-  blocked_to_striped_rev<32>(v, scratch, lane);      // the last level: the block merge's network
-  striped_stages<16>(v, c);
-  striped_to_blocked(v, scratch, 32, lane);
-  blocked_stages<true>(v, lane, c);
+#pragma unroll
+  for (int q = 0; q < CPR; ++q) sts128(sb + ((32 * q + lane) << 4), &v[q * E]);
 }
 
 template <typename KeyT, bool XIN>
@@ -135,53 +137,111 @@ __device__ __forceinline__ void cta_store_tile(const KeyT* src, KeyT* dst, int m
   for (int i = body + (int)threadIdx.x; i < m; i += blockDim.x) dst[i] = src[i];
 }
 
-// Everything after the load up to the sorted tile in shared memory: warp
-// sorts, then the CTA merge levels.  Returns the buffer (bufX or bufY of
-// smem_raw) that holds the tile's keys in order; its first min(T, n - base)
-// entries are the tile's.  xout: write the last level's output as floats.
+// Everything after the load: v (32 keys per lane, any assignment) to the sorted
+// tile in shared memory, first min(T, n - base) entries of the returned buffer.
+// Each lane sorts its 32 keys (a row).  Then a level merges pairs of sorted
+// blocks of 32h keys by one bitonic cascade -- strides of 32 and more between
+// registers in the striped layout, the rest inside the lane -- with h = 1 .. 16
+// inside each warp's 1024 keys and h = 32, 64, .. across the CTA:
+//   - warp levels come to the striped layout by a transpose in the warp's own
+//     part of the buffer that reads every second half backwards;
+//   - CTA levels by writing the blocks out in order and reading the window of
+//     the warp's output block (its co-ranks found by the merge-path search).
+// The tile is sorted in place in one buffer of 1024 * WARPS keys (aligned to
+// 1024 bytes): a barrier separates a CTA level's reads from its writes, and
+// half the shared memory lets four CTAs of 8-byte keys on an SM.  A short tile
+// is padded with the all-ones key (pads sort last, and one that ties with a
+// real key is bit-identical to it) and takes only the CTA levels its keys need.
+//
+// The levels are loops, not unrolled.  With 8-byte keys all of them share one
+// body: unrolled they were 161 KB of code, and a warp waited for its next
+// instruction longer than for anything else (2.05 of 6.5 warps per issue;
+// with four warps to a CTA no two warps of a scheduler run the same code at the
+// same time).  2 * 10^7 8-byte keys: 396 us unrolled, 279 us as one 49 KB body,
+// 262 us with every pair's second key taken from the sums (kTileMad64Pairs).
+// With 4-byte keys the warp levels and the CTA levels are a body each, and the
+// CTA levels use the directed last stages, which store in order at once:
+// 16.8 * 10^6 keys 117 us unrolled, 104 us as one body, 101 us as two, 98.5 us so.
+// Bound at that size: issue 69%, ALU 72%, shared-memory wavefronts 75% (4-byte), ALU 86%
+// before the sums (8-byte).
+// xout: write the last level's output as floats.
 template <typename KeyT, int WARPS>
 __device__ __forceinline__ KeyT* tile_sort_smem(KeyT (&v)[32], long long n, long long base,
                                                 bool xout, unsigned char* smem_raw) {
   constexpr int T = WARPS * kBlockItems;
-  KeyT* bufX = reinterpret_cast<KeyT*>(smem_raw);
-  KeyT* bufY = bufX + T + kTileSlack;
+  KeyT* buf = reinterpret_cast<KeyT*>(smem_raw);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  KeyT* own = buf + warp * kBlockItems;
+  const long long rem = n - base;
+  const int m = rem >= T ? T : (int)rem;
+  const TileMix c = mad_ones<TileMix>();
 
+  // From the striped layout, bitonic blocks of 2h rows, to sorted rows of the blocked layout.
+  auto network = [&](int h, auto flip) {
+    if (h >= 16) striped_stage<16>(v, c);            // strides 32h .. 32, at most 512
+    if (h >= 8) striped_stage<8>(v, c);
+    if (h >= 4) striped_stage<4>(v, c);
+    if (h >= 2) striped_stage<2>(v, c);
+    striped_stage<1>(v, c);
+    striped_to_blocked(v, own, 32, lane);
+    blocked_stages<decltype(flip)::value>(v, lane, c);   // strides 16 .. 1
+  };
+  auto to_floats = [&]() {
+#pragma unroll
+    for (int j = 0; j < 32; ++j) v[j] = (KeyT)ordered_to_f32((uint32_t)v[j]);
+  };
+  // Loads the window of the warp's block of the merge of sequences of len keys.
+  auto load_window = [&](int len) {
+    const int first = warp * kBlockItems & ~(2 * len - 1);   // the pair the block lies in
+    const int d0 = warp * kBlockItems - first;
+    const KeyT* A = buf + first;
+    const KeyT* B = A + len;
+    int a0, a1;
+    warp_corank_pair(A, len, B, len, d0, kBlockItems, lane, a0, a1);
+    warp_load_bitonic_full(A + a0, a1 - a0, B + (d0 - a0), v, lane);
+  };
+
+  lane_sort32(v, c);
   // The previous tile of a persistent CTA has been read out of shared memory
   // before the warps use it as transpose scratch.
   __syncthreads();
-  warp_sort_1024(v, bufX + warp * kBlockItems, lane);
-  if constexpr (WARPS == 1) {
-    warp_store_block<KeyT>(bufX, kBlockItems, v, lane, xout);
-    return bufX;
-  }
-  warp_store_block<KeyT>(bufX + warp * kBlockItems, kBlockItems, v, lane, false);
-  __syncthreads();
-
-  // CTA levels: merge the warps' sorted blocks pairwise up to the tile.
-  int my_off = lane * kBlockItems;
-  int my_len = 0;
-  {
-    const long long r2 = n - (base + (long long)lane * kBlockItems);
-    my_len = (lane < WARPS && r2 > 0) ? (r2 >= kBlockItems ? kBlockItems : (int)r2) : 0;
-  }
-  KeyT* src = bufX;
-  KeyT* dst = bufY;
-  int nseq = WARPS;
-  while (nseq > 1) {
-    cta_merge_level<KeyT, TileMix>(src, dst, my_off, my_len, nseq, warp, WARPS, lane,
-                                   xout && nseq <= 2);
-    next_seq<KeyT>(my_off, my_len, nseq, lane);
-    nseq = (nseq + 1) >> 1;
+  if constexpr (sizeof(KeyT) == 8) {
+#pragma unroll 1
+    for (int h = 1;; h *= 2) {
+      if (h <= 16) {
+        blocked_to_striped_rev(v, own, h, lane);
+      } else {
+        const bool last = 32 * h >= m;               // uniform over the CTA
+        blocked_to_linear(v, own, lane);
+        __syncthreads();
+        if (last) return buf;
+        load_window(32 * h);
+        __syncthreads();
+      }
+      network(h, std::false_type{});
+    }
+  } else {
+#pragma unroll 1
+    for (int h = 1; h <= 16; h *= 2) {
+      blocked_to_striped_rev(v, own, h, lane);
+      network(h, std::false_type{});
+    }
+    if (kBlockItems >= m && xout) to_floats();
+    blocked_to_linear(v, own, lane);
+#pragma unroll 1
+    for (int len = kBlockItems; len < m; len *= 2) {
+      __syncthreads();
+      load_window(len);
+      __syncthreads();
+      network(16, std::true_type{});
+      warp_store_block<KeyT>(own, kBlockItems, v, lane, xout && 2 * len >= m);
+    }
     __syncthreads();
-    KeyT* t = src;
-    src = dst;
-    dst = t;
+    return buf;
   }
-  return src;
 }
 
-// Everything after the load: the sort in shared memory and the store of the tile.
+// The sort in shared memory and the store of the tile.
 template <typename KeyT, int WARPS>
 __device__ __forceinline__ void tile_sort_finish(KeyT (&v)[32], KeyT* out, long long n,
                                                  long long base, bool xout,

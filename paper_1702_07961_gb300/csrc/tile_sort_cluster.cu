@@ -208,7 +208,7 @@ __global__ void __launch_bounds__(256, (MinBlocks<uint32_t, 8>::value))
 
 template <int CL, bool XIN, bool XOUT>
 static cudaError_t launch_cluster_t(const void* in, void* out, long long n, cudaStream_t s) {
-  const size_t smem = tile_sort_smem_bytes(4, 8);
+  const size_t smem = 2 * sizeof(uint32_t) * (size_t)(kCT + kTileSlack);   // two chunk buffers
   auto k = tile_sort_cluster_kernel<CL, XIN, XOUT>;
   cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
