@@ -40,6 +40,8 @@ struct SegPlan {
   int S;                  // tile items (base case and merge output tiles)
   int rounds;             // merge rounds launched
   int nphase;             // 1 + rounds
+  int kmax;               // largest fanout of the classes up to the declared maximum: what the
+                          // rounds' kernels are launched for
 };
 
 __host__ __device__ inline int size_class(unsigned long long n) {
@@ -96,7 +98,7 @@ __global__ void seg_plan_kernel(const unsigned long long* __restrict__ off, long
   }
   const long long tiles = (n + P.S - 1) / P.S;
   int K = P.class_fanout[size_class((unsigned long long)n)];
-  K = K < 2 ? 2 : (K > kMaxFanout ? kMaxFanout : K);
+  K = K < 2 ? 2 : (K > P.kmax ? P.kmax : K);
   int R = rounds_for(tiles, K);
   if (R > P.rounds) {
     set_device_error(dev_err, kDevErrInternal);   // a segment above the declared maximum
@@ -225,7 +227,10 @@ __global__ void __launch_bounds__(WARPS * 32, (TileMinBlocks<uint64_t, WARPS>::v
   }
 }
 
-template <typename KeyT>
+// K2MAX: the largest fanout of the batch's classes, rounded up to a power of
+// two (the code, and the registers, of larger ones are left out); Idx: int
+// when the whole batch is below 2^31 items.
+template <typename KeyT, int K2MAX, typename Idx>
 __global__ void __launch_bounds__(128)
     seg_splitter_kernel(const KeyT* bufA, const KeyT* bufB, const Desc* __restrict__ desc,
                         const int* __restrict__ total, long long per_phase, long long S, int r,
@@ -243,8 +248,18 @@ __global__ void __launch_bounds__(128)
       run_len *= K;
       tpg *= K;
     }
-    splitter_row<KeyT, 32>(in, (long long)d.n, run_len, K, S, idx / tpg, idx % tpg,
-                           table + t * kRowStride, 0xffffffffu, 0);
+    // tile counts fit 21 bits: the divisions need only 32
+    const unsigned tpg32 = tpg > 0xFFFFFFFFll ? 0xFFFFFFFFu : (unsigned)tpg;
+    const unsigned g = idx / tpg32, j = idx % tpg32;
+    long long* row = table + t * kRowStride;
+    const int k2 = pow2_ceil(K);                   // uniform over the warp
+    if (k2 == 2) splitter_row<KeyT, 2, Idx>(in, (long long)d.n, run_len, K, S, g, j, row);
+    if (k2 == 4) splitter_row<KeyT, 4, Idx>(in, (long long)d.n, run_len, K, S, g, j, row);
+    if (k2 == 8) splitter_row<KeyT, 8, Idx>(in, (long long)d.n, run_len, K, S, g, j, row);
+    if constexpr (K2MAX >= 16)
+      if (k2 == 16) splitter_row<KeyT, 16, Idx>(in, (long long)d.n, run_len, K, S, g, j, row);
+    if constexpr (K2MAX >= 32)
+      if (k2 == 32) splitter_row<KeyT, 32, Idx>(in, (long long)d.n, run_len, K, S, g, j, row);
   }
 }
 
@@ -443,17 +458,27 @@ cudaError_t launch_seg_tile_comp(const void* keys_in, void* a, void* b, const De
   return cudaGetLastError();
 }
 
-template <typename KeyT>
-cudaError_t launch_seg_split(const void* a, const void* b, const Desc* desc, const int* total,
-                             long long upper, long long S, int r, long long* table,
-                             cudaStream_t s) {
-  auto k = seg_splitter_kernel<KeyT>;
+template <typename KeyT, int K2MAX, typename Idx>
+cudaError_t launch_seg_split_t(const void* a, const void* b, const Desc* desc, const int* total,
+                               long long upper, long long S, int r, long long* table,
+                               cudaStream_t s) {
+  auto k = seg_splitter_kernel<KeyT, K2MAX, Idx>;
   unsigned grid = 1;
   cudaError_t e = persistent_grid(k, 128, 0, (upper + 3) / 4, &grid);
   if (e != cudaSuccess) return e;
   k<<<grid, 128, 0, s>>>(static_cast<const KeyT*>(a), static_cast<const KeyT*>(b), desc, total,
                          upper, S, r, table);
   return cudaGetLastError();
+}
+
+template <typename KeyT>
+cudaError_t launch_seg_split(const void* a, const void* b, const Desc* desc, const int* total,
+                             long long upper, long long S, int r, int kmax, bool small,
+                             long long* table, cudaStream_t s) {
+  if (!small) return launch_seg_split_t<KeyT, 32, long long>(a, b, desc, total, upper, S, r, table, s);
+  if (kmax <= 8) return launch_seg_split_t<KeyT, 8, int>(a, b, desc, total, upper, S, r, table, s);
+  if (kmax <= 16) return launch_seg_split_t<KeyT, 16, int>(a, b, desc, total, upper, S, r, table, s);
+  return launch_seg_split_t<KeyT, 32, int>(a, b, desc, total, upper, S, r, table, s);
 }
 
 template <typename KeyT, int WARPS>
@@ -500,18 +525,18 @@ cudaError_t seg_tile_phase(mms_key_type kt, bool pairs, int tw, const void* keys
   return cudaErrorInvalidValue;
 }
 
-cudaError_t seg_round(int unit_bytes, int tw, bool is_f32, int kmax, void* a, void* b,
+cudaError_t seg_round(int unit_bytes, int tw, bool is_f32, int kmax, bool small, void* a, void* b,
                       const Desc* desc, const int* total, long long upper, long long S, int r,
                       long long* table, int* dev_err, cudaStream_t s) {
   cudaError_t e;
   if (unit_bytes == 8) {
-    e = launch_seg_split<uint64_t>(a, b, desc, total, upper, S, r, table, s);
+    e = launch_seg_split<uint64_t>(a, b, desc, total, upper, S, r, kmax, small, table, s);
     if (e != cudaSuccess) return e;
     if (tw == 4) return launch_seg_merge<uint64_t, 4>(a, b, desc, total, upper, r, false, kmax, table, dev_err, s);
     if (tw == 2) return launch_seg_merge<uint64_t, 2>(a, b, desc, total, upper, r, false, kmax, table, dev_err, s);
     return cudaErrorInvalidValue;
   }
-  e = launch_seg_split<uint32_t>(a, b, desc, total, upper, S, r, table, s);
+  e = launch_seg_split<uint32_t>(a, b, desc, total, upper, S, r, kmax, small, table, s);
   if (e != cudaSuccess) return e;
   if (tw == 8) return launch_seg_merge<uint32_t, 8>(a, b, desc, total, upper, r, is_f32, kmax, table, dev_err, s);
   if (tw == 4) return launch_seg_merge<uint32_t, 4>(a, b, desc, total, upper, r, is_f32, kmax, table, dev_err, s);
@@ -667,6 +692,7 @@ static mms_status seg_sort_impl(mms_key_type kt, void* d_keys, uint32_t* d_value
   const int tw = P.S / 1024;
   int kmax = 2;
   for (int c = 0; c <= size_class(mx); ++c) kmax = P.class_fanout[c] > kmax ? P.class_fanout[c] : kmax;
+  P.kmax = kmax;
 
   if (prepare_only) return seg_prepare(kt, pairs, tw, kmax);
 
@@ -709,7 +735,7 @@ static mms_status seg_sort_impl(mms_key_type kt, void* d_keys, uint32_t* d_value
     st = chk(seg_tile_phase(kt, pairs, tw, d_keys, bufA, bufB, desc, totals, L.per_phase, s), "seg base case");
   mark();
   for (int r = 0; r < P.rounds && st == MMS_OK; ++r) {
-    st = chk(seg_round(unit, tw, kt == MMS_KEY_F32 && !pairs, kmax, bufA, bufB,
+    st = chk(seg_round(unit, tw, kt == MMS_KEY_F32 && !pairs, kmax, total_n < (1ull << 31), bufA, bufB,
                        desc + (long long)(1 + r) * L.per_phase, totals + 1 + r, L.per_phase, P.S,
                        r, table, dev_err, s),
              "seg merge round");

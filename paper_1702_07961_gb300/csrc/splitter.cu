@@ -4,52 +4,65 @@
 
 namespace mms {
 
-// Warps per splitter CTA: 4 measured fastest on GB300 at 10^8 u32 keys
-// (splitters 0.302 ms, against 0.306 with 2 warps and 0.307 with 8).
+// Warps per splitter CTA: on GB300 2 and 4 measure the same, 8 is 1 to 3%
+// slower (10^8 u32 keys, and 2 * 10^7 u64).
 constexpr int kSplitterWarps = 4;
 
-template <typename KeyT, int W, typename Idx>
+// Rows up to which the splitter is launched with programmatic stream serialization.
+// Behind a merge pass it then starts on SMs whose memory is set up as shared
+// memory, and a row's samples of a step do not fit the L1 that is left: from
+// 2^23 keys on the gap saved costs more than it gives (10^8 u32 keys 2669 -> 2539
+// us without it, 16.8 * 10^6 451 -> 404, 2^23 256 -> 215; 2^21 93 either way; 2^20 78
+// without, 66 with).
+constexpr long long kSplitterPdlTiles = 192;
+
+template <typename KeyT, int K2, typename Idx>
 __global__ void __launch_bounds__(32 * kSplitterWarps)
     splitter_kernel(const KeyT* __restrict__ in, long long n, long long run_len, int K,
-                    long long S, long long tpg, long long ntiles, long long* __restrict__ table) {
-  const int lane = threadIdx.x & 31;
-  const int gb = lane & ~(W - 1);                 // first lane of this lane group
-  const unsigned gm = W == 32 ? 0xffffffffu : (((1u << W) - 1u) << gb);
+                    long long S, unsigned tpg, unsigned ntiles, long long* __restrict__ table) {
   griddep_wait();                                 // the runs are the previous kernel's output
   griddep_launch_dependents();
-  const long long t = ((long long)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5)) * (32 / W) + gb / W;
-  if (t >= ntiles) return;                        // uniform over the lane group
-  splitter_row<KeyT, W, Idx>(in, n, run_len, K, S, t / tpg, t % tpg, table + t * K, gm, gb);
+  const unsigned t = blockIdx.x * kSplitterWarps + (threadIdx.x >> 5);
+  if (t >= ntiles) return;                        // uniform over the warp
+  splitter_row<KeyT, K2, Idx>(in, n, run_len, K, S, t / tpg, t % tpg, table + (long long)t * K);
 }
 
-template <typename KeyT, int W>
-static cudaError_t launch_w(const void* in, long long n, long long run_len, int K, long long S,
-                            long long tpg, long long ntiles, long long* table, cudaStream_t s,
-                            bool pdl) {
-  const long long per_block = kSplitterWarps * (32 / W);   // warps of 32 / W tiles each
-  const unsigned grid = (unsigned)((ntiles + per_block - 1) / per_block);
+template <typename KeyT, int K2>
+static cudaError_t launch_k2(const void* in, long long n, long long run_len, int K, long long S,
+                             unsigned tpg, unsigned ntiles, long long* table, cudaStream_t s,
+                             bool pdl) {
+  const unsigned grid = (ntiles + kSplitterWarps - 1) / kSplitterWarps;
   const KeyT* kin = static_cast<const KeyT*>(in);
-  // 32-bit counts and positions while no probe can pass 2^31 (n < 2^30)
-  if (n < (1ll << 30))
-    return launch_k(splitter_kernel<KeyT, W, int>, dim3(grid), dim3(32 * kSplitterWarps), 0, s, pdl, kin, n, run_len,
+  if (n < (1ll << 31))                            // counts and positions fit 32 bits
+    return launch_k(splitter_kernel<KeyT, K2, int>, dim3(grid), dim3(32 * kSplitterWarps), 0, s, pdl, kin, n, run_len,
                     K, S, tpg, ntiles, table);
-  return launch_k(splitter_kernel<KeyT, W, long long>, dim3(grid), dim3(32 * kSplitterWarps), 0, s, pdl, kin, n,
+  return launch_k(splitter_kernel<KeyT, K2, long long>, dim3(grid), dim3(32 * kSplitterWarps), 0, s, pdl, kin, n,
                   run_len, K, S, tpg, ntiles, table);
 }
 
-// One output tile per warp (W = 32).  Packing 32 / W tiles into a warp's lane
-// groups was measured slower on GB300 (10^8 u32: 0.65 ms of splitters at
-// K = 4 against 0.47 ms): the search is bound by the latency of its
-// dependent loads and needs the independent warps, and lane groups of one
-// warp diverge in their per-tile pop loops.
+template <typename KeyT>
+static cudaError_t launch_key(const void* in, long long n, long long run_len, int K, long long S,
+                              unsigned tpg, unsigned ntiles, long long* table, cudaStream_t s, bool pdl) {
+  switch (pow2_ceil(K)) {
+    case 2: return launch_k2<KeyT, 2>(in, n, run_len, K, S, tpg, ntiles, table, s, pdl);
+    case 4: return launch_k2<KeyT, 4>(in, n, run_len, K, S, tpg, ntiles, table, s, pdl);
+    case 8: return launch_k2<KeyT, 8>(in, n, run_len, K, S, tpg, ntiles, table, s, pdl);
+    case 16: return launch_k2<KeyT, 16>(in, n, run_len, K, S, tpg, ntiles, table, s, pdl);
+    default: return launch_k2<KeyT, 32>(in, n, run_len, K, S, tpg, ntiles, table, s, pdl);
+  }
+}
+
+// One output tile per warp.
 cudaError_t launch_splitter(int key_bytes, long long S, const void* in, long long n,
                             long long run_len, int K, long long* table, cudaStream_t s, bool pdl) {
   const long long ntiles = num_tiles(S, n, run_len, K);
   if (ntiles <= 0) return cudaSuccess;
-  if (K < 2 || K > kMaxFanout) return cudaErrorInvalidValue;
-  const long long tpg = tiles_per_group(S, run_len, K);
-  if (key_bytes == 4) return launch_w<uint32_t, 32>(in, n, run_len, K, S, tpg, ntiles, table, s, pdl);
-  return launch_w<uint64_t, 32>(in, n, run_len, K, S, tpg, ntiles, table, s, pdl);
+  if (K < 2 || K > kMaxFanout || ntiles > 0x7FFFFFFFll) return cudaErrorInvalidValue;
+  if (ntiles > kSplitterPdlTiles) pdl = false;
+  long long tpg = tiles_per_group(S, run_len, K);
+  if (tpg > 0xFFFFFFFFll) tpg = 0xFFFFFFFFll;     // more than the grid: every tile is in group 0
+  if (key_bytes == 4) return launch_key<uint32_t>(in, n, run_len, K, S, (unsigned)tpg, (unsigned)ntiles, table, s, pdl);
+  return launch_key<uint64_t>(in, n, run_len, K, S, (unsigned)tpg, (unsigned)ntiles, table, s, pdl);
 }
 
 }  // namespace mms

@@ -239,27 +239,191 @@ __device__ __forceinline__ Idx multiseq_pivot(const KeyT* run, Idx rlen, bool ac
   return d;
 }
 
-// Pivots of output tile j of group g, found by one lane group of W >= K lanes
-// (gm: its lanes, gb: its first lane; lane gb + r handles run r): row[r]
-// receives the number of items of run r among the group's first j * S
-// outputs.  Arguments are uniform over the lane group.  Idx is the type of
-// the counts and positions of the search: int when n < 2^30 (every position
-// probed stays below 2n), long long otherwise.
-template <typename KeyT, int W, typename Idx = long long>
+// The search of the splitter kernels: the same pivots by the same idea --
+// exact pivots of the s-sample problem, s shrinking to 1 -- but with a window
+// of W samples of every run held across the warp, so that a step divides s by
+// W / 2 instead of 2 and its drops are found together, not one arg-max at a
+// time.  One warp per row.  SUB = 32 / K2 lanes share a run (K2: K rounded up
+// to a power of two); register m of sub-lane b holds the sample
+// f = top - W + 1 + b * M + m of the run, counted from 1, which is the item at
+// position f * s - 1.
+//
+//   - Let c be the run's pivot at stride s' = s * W / 2, exact for the rank
+//     floor(k / s').  Sample c + 1 of stride s' was left out there, so at least
+//     floor(k / s') + 1 samples of stride s' come no later, each with W / 2 samples
+//     of stride s at or below it: more than floor(k / s).  So the pivot at
+//     stride s is at most top = min(c * W / 2 + W / 2 - 1, len / s).
+//   - D = max(0, sum of the tops - floor(k / s)) samples must go, the largest
+//     ones.  The 32 M windowed samples are sorted across the warp (bitonic
+//     merges of the windows, which are sorted already); the D-th largest is the
+//     threshold, and every lane compares its own samples with it.
+//   - A run whose whole window goes may have to give up more.  Of those runs
+//     the one whose lowest windowed sample is the largest loses its whole
+//     window for certain (samples not yet seen are all smaller), so it moves
+//     on by one window and the selection is repeated with D - W.  About 3% of
+//     the steps of 16 random runs do this, fewer with fewer runs.
+//   - The first stride is the least power of W / 2 at which every run has at most W
+//     samples; there top = len / s and the windows are all there is.
+//
+// Ties are broken by (run, position), so the pivots are those of multiseq_pivot.
+//
+// What bounds it: up to about 3000 rows (one wave of warps) a chain of
+// log(run_len) / log(W / 2) steps, each a load (700 cycles and more) and a sort of
+// about as long; above that the 32 M sectors a step reads.  Stride halving took
+// log2(K * run_len) levels, each a load and about K / 2 arg-maxes of 250 cycles.  Both
+// splitters of 2^20 u32 keys 41 -> 25 us, the three of 16.8 * 10^6 85 -> 59 us, the
+// four of 10^8 304 -> 264 us.  Finding the threshold by quickselect instead of
+// sorting took 500 cycles a round of 5 to 7 rounds and was no faster than stride halving.
+
+// Samples per lane.  More samples take fewer, longer steps and read more
+// sectors: with K = 8, 4 against 2 measured 12.3 against 18.4 us at 2^20 u32 keys and
+// 62 against 70 us at 10^8; with K = 4, 1 against 4 18.5 against 28.5 us at 2 * 10^7 u64.
+__host__ __device__ constexpr int pivot_regs(int k2) {
+  return k2 == 32 ? 8 : k2 >= 8 ? 4 : 1;
+}
+
+// One bitonic merge level: sorted sequences of N / 2 elements become sorted ones of
+// N, element e of the warp in register e % M of lane e / M, all ascending.  The
+// first stage compares e with its mirror image in the block of N.
+template <int N, int M, typename KeyT>
+__device__ __forceinline__ void window_merge(KeyT (&v)[M], int lane) {
+  KeyT y[M];
+#pragma unroll
+  for (int s = N / 2; s >= 1; s >>= 1) {
+    if (s >= M) {                                  // between lanes
+      const bool upper = (lane & (s / M)) != 0;
+#pragma unroll
+      for (int m = 0; m < M; ++m)
+        y[m] = s == N / 2 ? __shfl_xor_sync(0xffffffffu, v[M - 1 - m], N / M - 1)
+                          : __shfl_xor_sync(0xffffffffu, v[m], s / M);
+#pragma unroll
+      for (int m = 0; m < M; ++m) v[m] = (y[m] < v[m]) != upper ? y[m] : v[m];
+    } else {
+#pragma unroll
+      for (int m = 0; m < M; ++m)
+        if ((m & s) == 0) cas(v[m], v[m + s]);
+    }
+  }
+}
+
+// Sorted sequences of N elements to one of 32 M.
+template <int N, int M, typename KeyT>
+__device__ __forceinline__ void window_sort(KeyT (&v)[M], int lane) {
+  if constexpr (N < 32 * M) {
+    window_merge<2 * N, M>(v, lane);
+    window_sort<2 * N, M>(v, lane);
+  }
+}
+
+// `run` and `rlen`: the run of this lane (lane / SUB) and its length, 0 past
+// the K runs; maxlen: an upper bound of the lengths; k <= their sum.  All 32
+// lanes call, k and maxlen uniform.  Returns the run's pivot on each of its
+// lanes.  Idx as for multiseq_pivot (positions never pass the run's end).
+template <typename KeyT, int K2, typename Idx>
+__device__ __forceinline__ Idx window_pivot(const KeyT* run, Idx rlen, Idx maxlen, Idx k) {
+  constexpr int SUB = 32 / K2;
+  constexpr int M = pivot_regs(K2);
+  constexpr int W = SUB * M;
+  constexpr int B = W == 4 ? 1 : W == 8 ? 2 : W == 16 ? 3 : W == 32 ? 4 : 5;   // log2(W / 2)
+  static_assert(W == (2 << B), "windows of 4 to 64 samples");
+  const int lane = threadIdx.x & 31, sub = lane % SUB;
+  if (k == 0) return 0;
+  int sh = 0;
+  while ((maxlen >> sh) > W) sh += B;
+  Idx top = rlen >> sh;
+  for (;;) {
+    int D = (int)(__reduce_add_sync(0xffffffffu, sub == 0 ? (unsigned)top : 0u) - (unsigned)(k >> sh));
+    int gone = 0;
+    while (D > 0) {
+      KeyT w[M], v[M];
+      int tot = 0;
+#pragma unroll
+      for (int m = 0; m < M; ++m) {
+        const Idx f = top - (Idx)(W - 1 - m - sub * M);
+        w[m] = f >= 1 ? run[(f << sh) - 1] : KeyT(0);
+        v[m] = w[m];
+        tot += __popc(__ballot_sync(0xffffffffu, f >= 1));
+      }
+      unsigned X[M];
+      if (D >= tot) {                              // everything in the windows goes
+#pragma unroll
+        for (int m = 0; m < M; ++m) X[m] = __ballot_sync(0xffffffffu, top >= (Idx)(W - m - sub * M));
+      } else {
+        window_sort<W, M>(v, lane);
+        const int pos = 32 * M - D;                // the D largest start there
+        KeyT t = v[0];
+#pragma unroll
+        for (int m = 1; m < M; ++m) t = pos % M == m ? v[m] : t;
+        t = __shfl_sync(0xffffffffu, t, pos / M);
+        unsigned E[M];
+        int need = D, eq = 0;
+#pragma unroll
+        for (int m = 0; m < M; ++m) {
+          X[m] = __ballot_sync(0xffffffffu, w[m] > t);
+          E[m] = __ballot_sync(0xffffffffu, w[m] == t && top >= (Idx)(W - m - sub * M));
+          need -= __popc(X[m]);
+          eq += __popc(E[m]);
+        }
+        if (need == eq) {
+#pragma unroll
+          for (int m = 0; m < M; ++m) X[m] |= E[m];
+        } else {                                   // of equal keys, those of the later runs and places
+          int above = 0;
+#pragma unroll
+          for (int m = 0; m < M; ++m) above += __popc(E[m] & ~(0xffffffffu >> (31 - lane)));
+#pragma unroll
+          for (int m = M - 1; m >= 0; --m) {
+            const bool mine = (E[m] >> lane) & 1u;
+            X[m] |= __ballot_sync(0xffffffffu, mine && above < need);
+            above += mine;
+          }
+        }
+      }
+      gone = 0;
+#pragma unroll
+      for (int m = 0; m < M; ++m) gone += __popc((X[m] >> (lane - sub)) & (unsigned)((1ull << SUB) - 1));
+      const bool deep = sub == 0 && gone == W && top > W;   // its lane holds the lowest sample
+      if (!__any_sync(0xffffffffu, deep)) break;
+      const int r = (31 - __clz(lanes_with_max(0xffffffffu, deep, w[0]))) / SUB;
+      if (lane / SUB == r) top -= W;
+      D -= W;
+      gone = 0;
+    }
+    top -= gone;
+    if (sh == 0) return top;
+    sh -= B;
+    const Idx cap = rlen >> sh;
+    top = (top << B) + ((1 << B) - 1);
+    top = top < cap ? top : cap;
+  }
+}
+
+// Pivots of output tile j of group g, found by one warp: row[r] receives the
+// number of items of run r among the group's first j * S outputs.  Arguments
+// are uniform over the warp.  Idx is the type of the counts and positions of
+// the search: int when n < 2^31, long long otherwise.  K2: K rounded up to a power of two.
+template <typename KeyT, int K2, typename Idx = long long>
 __device__ __forceinline__ void splitter_row(const KeyT* __restrict__ in, long long n,
                                              long long run_len, int K, long long S, long long g,
-                                             long long j, long long* __restrict__ row,
-                                             unsigned gm, int gb) {
+                                             long long j, long long* __restrict__ row) {
+  constexpr int SUB = 32 / K2;
   const int lane = threadIdx.x & 31;
-  const int rr = lane - gb;                     // run of this lane
+  const int rr = lane / SUB;                    // run of this lane
   const bool act = rr < K;
   const long long rstart = g * run_len * K + (long long)rr * run_len;
   long long rlen64 = n - rstart;
   rlen64 = rlen64 < 0 ? 0 : (rlen64 > run_len ? run_len : rlen64);
   const Idx rlen = act ? (Idx)rlen64 : Idx(0);
   const KeyT* run = in + (act ? rstart : 0);
-  const Idx d = multiseq_pivot<KeyT, Idx, true>(run, rlen, act, K, (Idx)(j * S), gm);
-  if (act) row[rr] = d;
+  const Idx d = window_pivot<KeyT, K2, Idx>(run, rlen, (Idx)(run_len < n ? run_len : n), (Idx)(j * S));
+  if (act && lane % SUB == 0) row[rr] = d;
+}
+
+// K rounded up to a power of two (K in 2..32), for the dispatch on K2.
+__host__ __device__ inline int pow2_ceil(int K) {
+  int k2 = 2;
+  while (k2 < K) k2 *= 2;
+  return k2;
 }
 
 }  // namespace mms
