@@ -22,6 +22,10 @@ def runs_of(kind, K, run_len, last, dtype, seed):
             x = g.integers(900, 1000, n) if r == K // 2 else g.integers(0, 1000, n)
         elif kind == "disjoint up":
             x = r * run_len + np.arange(n)
+        elif kind == "nearly sorted":  # disjoint runs but for one sample in ten, which lies anywhere
+            x = np.where(g.random(n) < 0.1, g.integers(0, K * run_len, n), r * run_len + np.arange(n))
+        elif kind == "two dense":      # two runs hold the upper values, with ties
+            x = g.integers(990, 1000, n) if r in (1, K // 2 + 1) else g.integers(0, 1000, n)
         elif kind == "disjoint down":
             x = (K - r) * run_len + np.arange(n)
         else:                         # "ties": two values, the largest key among them
@@ -31,7 +35,7 @@ def runs_of(kind, K, run_len, last, dtype, seed):
 
 
 @pytest.mark.parametrize("dtype", [np.uint32, np.uint64])
-@pytest.mark.parametrize("kind", ["scales", "one dense", "disjoint up", "disjoint down", "ties"])
+@pytest.mark.parametrize("kind", ["scales", "one dense", "two dense", "disjoint up", "disjoint down", "nearly sorted", "ties"])
 @pytest.mark.parametrize("K,mult", [(2, 1), (5, 3), (8, 1), (11, 2), (16, 1), (27, 1), (32, 2)])
 def test_tables(gpu, dtype, kind, K, mult):
     import torch
