@@ -48,7 +48,7 @@ __device__ __forceinline__ bool consumers_any(bool v) {
 
 template <typename KeyT, int WARPS>
 struct PipeGeom {
-  static constexpr int kCtlInts = (int)(kMergeCtlBytes / sizeof(int));
+  static constexpr int kCtlStride = (int)(kMergeCtlBytes / sizeof(int));
   __host__ __device__ static constexpr size_t buf_bytes(int K) {
     return sizeof(KeyT) * (size_t)MergeGeom<KeyT, WARPS>::cap(K);   // a multiple of 16
   }
@@ -103,12 +103,12 @@ __global__ void __launch_bounds__((WARPS + 1) * 32, 2)
       const long long g = t / tpg, j = t % tpg;
       long long lo = 0, hi = 0;
       merge_tile_pivots(n, run_len, K, g, j, table + t * K, table + (t + 1) * K, S, lane, lo, hi);
-      int* ctl = ctls + b * P::kCtlInts;
+      int* ctl = ctls + b * P::kCtlStride;
       merge_plan_warp<KeyT, WARPS>(in, n, run_len, K, g, j, lo, hi, S, buf(b), ctl, &full[b], lane);
       __syncwarp();
       if (lane == 0) {
         // A rejected plan started no copies and made no expect-tx arrival.
-        if (ctl[kCtlNodeFields * 32 + 3]) mbar_arrive_plain(&full[b]);
+        if (ctl[kCtlErr]) mbar_arrive_plain(&full[b]);
         mbar_arrive_plain(&full[b]);              // publishes the node table and plain loads
       }
       staged = q + 1;
@@ -136,9 +136,9 @@ __global__ void __launch_bounds__((WARPS + 1) * 32, 2)
       if (threadIdx.x == 0) set_device_error(dev_err, kDevErrTimeout);
       return;                                     // uniform over the merging warps
     }
-    const int* ctl = ctls + b * P::kCtlInts;
+    const int* ctl = ctls + b * P::kCtlStride;
     const long long g = t / tpg, j = t % tpg;
-    if (ctl[kCtlNodeFields * 32 + 3]) {
+    if (ctl[kCtlErr]) {
       if (threadIdx.x == 0) set_device_error(dev_err, kDevErrInternal);
     } else {
       merge_levels<KeyT, WARPS>(buf(b), buf(p), ctl, out + g * run_len * K + j * S, XOUT,

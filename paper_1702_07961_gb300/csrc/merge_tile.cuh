@@ -32,30 +32,41 @@
 
 namespace mms {
 
-// Control area after a merge CTA's mbarrier: the merge-tree node table (10
-// fields x 32 nodes) and four scalars, written by warp 0 for the whole CTA.
-constexpr int kCtlNodeFields = 10;
-constexpr int kCtlScalars = 8;
-constexpr size_t kMergeCtlBytes = sizeof(int) * (kCtlNodeFields * 32 + kCtlScalars);
+// Control area after a merge CTA's mbarrier, written by the planning warps for
+// the whole CTA (ints): four scalars, four per tree level (its first item, the
+// end of its network items, the end of its items, unused), and the items, 16
+// bytes each.  An item is one output block of a node:
+//   x: offset of the node's sequence A | its length << 16,   y: the same of B,
+//   z: offset of the node's output | the block's start in it << 16,   w: the block's size.
+constexpr int kCtlLevels = 0, kCtlWant = 2, kCtlErr = 3;
+constexpr int kCtlLevel0 = 4;                        // level lv at kCtlLevel0 + 4 * lv
+constexpr int kCtlItems = 32;
+constexpr int kMaxItems = 72;                        // 71 at most: 8 per level, and one per node, with K = 32
+constexpr int kCtlInts = kCtlItems + 4 * kMaxItems;
+constexpr size_t kMergeCtlBytes = sizeof(int) * kCtlInts;
 
 // Shared-memory geometry of a merge CTA for fanout K.  X: the staged
 // segments, each at a 16-byte aligned span start R_r (up to 2E-2 items of
-// alignment slack and 32 items of transpose slack per segment), and the odd
-// tree levels' inputs; Y: the same spans, one buffer per level parity.
+// alignment slack and 16 items of transpose slack per segment: a node that runs a
+// network has two segments at least, and its last block may use 31 items past
+// its end), and the odd tree levels' inputs; Y: the same spans, one buffer per
+// level parity.  Three CTAs fit an SM up to K = 32 (76464 of 76800 bytes with 8-byte keys).
 template <typename KeyT, int WARPS>
 struct MergeGeom {
   static constexpr int E = Vec16<KeyT>::E;
   static constexpr int S = WARPS * kBlockItems;
-  static constexpr int kSlack = 32;
-  __host__ __device__ static constexpr int cap(int K) { return S + K * (2 * E + kSlack) + E; }
-  // control block: mbarrier (16 bytes with padding), then the node table
+  static constexpr int kSlack = 16;
+  __host__ __device__ static constexpr int cap(int K) {
+    return S + (K * (2 * E - 2 + kSlack) + E - 1) / E * E + E;
+  }
+  // control block: mbarrier (16 bytes with padding), then the control area
   __host__ __device__ static constexpr size_t bytes(int K) {
     return sizeof(KeyT) * 2 * (size_t)cap(K) + 16 + kMergeCtlBytes;
   }
-  // The partition variant adds its pivot rows after the control area: row b
-  // (b <= WARPS) holds, per segment, the items of the tile's first 1024 b
-  // outputs.
-  static constexpr size_t kRowBytes = sizeof(int) * 32 * (WARPS + 1);
+  // The partition variant adds, after the control area, the offset and the length of every
+  // staged segment and its pivot rows: row b (b <= WARPS) holds, per segment,
+  // the items of the tile's first 1024 b outputs.
+  static constexpr size_t kRowBytes = sizeof(int) * 32 * (WARPS + 3);
   __host__ __device__ static constexpr size_t bytes_partition(int K) { return bytes(K) + kRowBytes; }
 };
 
@@ -98,14 +109,14 @@ __device__ __forceinline__ void merge_tile_pivots(long long n, long long run_len
 // Plans output tile j of group g, whose segment bounds in run `lane` are lo
 // and hi (from merge_tile_pivots), and stages its segments into `stage`: one
 // warp, one lane per run and one per merge-tree node.  Starts the bulk copies
-// on `bar`, loads the items no bulk copy covers, and writes the node table and
-// the scalars (levels, nodes, tile size, error) into `ctl`; the caller's CTA
+// on `bar`, loads the items no bulk copy covers, and writes the items and
+// the scalars (levels, tile size, error) into `ctl`; the caller's CTA
 // barrier publishes the plain loads and the table, the barrier's phase the
 // copies.  On segment bounds that fail their check, ctl's error scalar is set
 // and nothing is staged.
 // `part` splits the work between two warps that both call this with the same
 // bounds: bit 0 stages the segments (and writes the tile size and error
-// scalars), bit 1 writes the node table (and the level and node counts).  The
+// scalars), bit 1 writes the items (and the levels' bounds).  The
 // two halves need only the segment lengths and spans, which both compute, so a
 // CTA can start the copies and build the table at the same time.
 template <typename KeyT, int WARPS>
@@ -113,7 +124,7 @@ __device__ __forceinline__ void merge_plan_warp(const KeyT* __restrict__ in, lon
                                                 long long run_len, int K, long long g,
                                                 long long j, long long lo, long long hi, int S,
                                                 KeyT* stage, int* ctl, uint64_t* bar, int lane,
-                                                int part = 3) {
+                                                int part = 3, int* segs = nullptr) {
   using G = MergeGeom<KeyT, WARPS>;
   constexpr int E = G::E;
   const long long gstart = g * run_len * K;
@@ -133,8 +144,8 @@ __device__ __forceinline__ void merge_plan_warp(const KeyT* __restrict__ in, lon
   const bool bad = __any_sync(0xffffffffu, bad_seg) || sum != want || K > kMaxFanout || K < 2 ||
                    S > G::S || S < kBlockItems || (smem_u32addr(stage) & 15u) != 0;
   if (lane == 0 && (part & 1)) {
-    ctl[kCtlNodeFields * 32 + 2] = (int)want;
-    ctl[kCtlNodeFields * 32 + 3] = bad ? 1 : 0;
+    ctl[kCtlWant] = (int)want;
+    ctl[kCtlErr] = bad ? 1 : 0;
   }
   if (!bad) {
     const long long gsrc = rstart + lo;              // first item, index into `in`
@@ -189,6 +200,10 @@ __device__ __forceinline__ void merge_plan_warp(const KeyT* __restrict__ in, lon
       if (__any_sync(0xffffffffu, act && len > 0 && bulk_hi < gsrc + len)) plain_tail();
     }
     if (!(part & 2)) return;
+    if (segs != nullptr) {                           // for the partition variant
+      segs[lane] = R + head;
+      segs[32 + lane] = len;
+    }
     // Merge-tree nodes, one per lane, in level order: node (level l >= 1,
     // pair q) merges child A = segments [q*2^l, q*2^l + 2^(l-1)) and child
     // B = the rest of [q*2^l, (q+1)*2^l) (segments past the group's runs are
@@ -233,15 +248,16 @@ __device__ __forceinline__ void merge_plan_warp(const KeyT* __restrict__ in, lon
     // A node's last block is "small" when it holds at most kSmallBlockMax
     // items; it is merged by the small network, after every full-size block
     // of its level, so that the level's big blocks are dealt first and the
-    // cheap ones fill in.  Work items of a level: its nodes' big blocks in
-    // node order, then its small blocks in node order; levels follow each
-    // other.  Inclusive scans over the nodes (lanes, in level order) of the
-    // big and the small block counts give every node its first big item and
-    // its small item: with n0 / n1 the first / last node of the node's level,
-    //   first big item = big blocks before the node + small blocks before n0,
-    //   small item     = big blocks up to n1 + small blocks before the node.
+    // cheap ones fill in.  So are the blocks of a node with an empty child, which
+    // are copies.  Items of a level: its nodes' big blocks in node order,
+    // then the others in node order; levels follow each other.
+    // Inclusive scans over the nodes (lanes, in level order) of both counts
+    // give every node its first item of each kind: with n0 / n1 the first /
+    // last node of the node's level,
+    //   first big item = big blocks before the node + others before n0,
+    //   first other    = big blocks up to n1 + others before the node.
     const int tail = lenA + lenB - (nb - 1) * kBlockItems;
-    const int small = (nb > 0 && tail <= kSmallBlockMax) ? 1 : 0;
+    const int small = (lenA == 0 || lenB == 0) ? nb : (nb > 0 && tail <= kSmallBlockMax) ? 1 : 0;
     const int nbig = nb - small;
     int sbig = nbig, ssm = small;
 #pragma unroll
@@ -258,97 +274,156 @@ __device__ __forceinline__ void merge_plan_warp(const KeyT* __restrict__ in, lon
     const int small_before_n0 = __shfl_sync(0xffffffffu, ssm - small, n0);
     const int big_upto_n1 = __shfl_sync(0xffffffffu, sbig, n1);
     const int small_upto_n1 = __shfl_sync(0xffffffffu, ssm, n1);
-    ctl[0 * 32 + lane] = lenA;
-    ctl[1 * 32 + lane] = lenB;
-    ctl[2 * 32 + lane] = (c_level == 1) ? rf + hf : rf;                     // staged segment
-    ctl[3 * 32 + lane] = (mid < K) ? ((c_level == 1) ? rm + hm : rm) : 0;   // vs. child output
-    ctl[4 * 32 + lane] = rf;                                                // output span
-    ctl[5 * 32 + lane] = (sbig - nbig) + small_before_n0;                  // first big item
-    ctl[6 * 32 + lane] = nb;
-    ctl[7 * 32 + lane] = is_node ? c_level : 0;
-    ctl[8 * 32 + lane] = small ? big_upto_n1 + (ssm - small) : -1;         // small item
-    ctl[9 * 32 + lane] = big_upto_n1 + small_upto_n1;                      // end of the level
-    if (lane == 0) {
-      ctl[kCtlNodeFields * 32 + 0] = nl;
-      ctl[kCtlNodeFields * 32 + 1] = nnodes;
+    const int offA = (c_level == 1) ? rf + hf : rf;                      // staged segment
+    const int offB = (mid < K) ? ((c_level == 1) ? rm + hm : rm) : 0;    // vs. child output
+    const int first_big = (sbig - nbig) + small_before_n0;
+    const int first_other = big_upto_n1 + (ssm - small);
+    if (is_node) {
+      int4* items = reinterpret_cast<int4*>(ctl + kCtlItems);
+      for (int blk = 0; blk < nb; ++blk) {
+        const int at = blk < nbig ? first_big + blk : first_other + (blk - nbig);
+        const int left = lenA + lenB - blk * kBlockItems;
+        if (at < kMaxItems)
+          items[at] = make_int4(offA | (lenA << 16), offB | (lenB << 16), rf | ((blk * kBlockItems) << 16),
+                                left < kBlockItems ? left : kBlockItems);
+      }
+      if (lane == n0) {
+        int* lv = ctl + kCtlLevel0 + 4 * c_level;
+        lv[0] = first_big;
+        lv[2] = big_upto_n1 + small_upto_n1;
+      }
+      if (lane == n1) ctl[kCtlLevel0 + 4 * c_level + 1] = first_big + nbig;
     }
+    if (lane == 0) ctl[kCtlLevels] = nl;
   }
 }
 
 // Merges a staged tile level by level and writes it to dstg: run by the
 // WARPS merging warps (threads 0 .. 32 * WARPS - 1).  bufX holds the staged
-// segments, bufY is the other level buffer; `ctl` is the tile's node table.
+// segments, bufY is the other level buffer; `ctl` is the tile's control area.
 // sync() is a barrier over exactly the merging warps; the caller has made the
-// staged data and the table visible to them.
+// staged data and the control area visible to them.
+//
+// A level's items are dealt to the warps round-robin: first the network
+// items, then the small and the copied blocks; a barrier ends the level.  Each
+// lane reads the item's 16 bytes (in place of the ballots and shuffles that looked a
+// node up: 350 cycles of an item's 3500 with one CTA on the SM).
+//
+// The last stages of a block run in the blocked layout.  It leaves it in order:
+// the rows go to their place swizzled, come back as consecutive 16-byte chunks, and
+// are stored once more -- or, where the root's blocks are all network items and the
+// tile lies on the 16-byte grid, straight to global memory, with no barrier,
+// bulk store and wait after them: passes of 16.8 * 10^6 u32 keys 37.1 / 54.3 / 73.4 /
+// 92.3 us to 35.0 / 52.3 / 71.0 / 89.9 (K = 2, 4, 8, 16; K = 32, now three CTAs to an SM,
+// 149.9 to 122.3).  With 8-byte keys the last stages are directed
+// instead (a compare's predicate takes a direction for nothing), which stores in
+// place at once; their tile goes out by the bulk store.
 template <typename KeyT, int WARPS, typename Sync>
 __device__ __forceinline__ void merge_levels(KeyT* bufX, KeyT* bufY, const int* ctl,
                                              KeyT* __restrict__ dstg, bool xout, Sync sync) {
   constexpr int E = Vec16<KeyT>::E;
+  constexpr uint32_t RB = 32 * sizeof(KeyT);
+  constexpr bool LINEAR = sizeof(KeyT) == 4;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int nl = ctl[kCtlNodeFields * 32 + 0];
-  const int nnodes = ctl[kCtlNodeFields * 32 + 1];
-  const long long want = ctl[kCtlNodeFields * 32 + 2];
-  const bool is_node = lane < nnodes;
-  const int c_lenA = ctl[0 * 32 + lane], c_lenB = ctl[1 * 32 + lane];
-  const int c_offA = ctl[2 * 32 + lane], c_offB = ctl[3 * 32 + lane];
-  const int c_out = ctl[4 * 32 + lane], c_first = ctl[5 * 32 + lane];
-  const int c_nb = ctl[6 * 32 + lane], c_level = ctl[7 * 32 + lane];
-  const int c_small = ctl[8 * 32 + lane], c_end = ctl[9 * 32 + lane];
-  const int c_nbig = c_nb - (c_small >= 0 ? 1 : 0);
-
-  // Level by level: the big blocks of the level's nodes, then their small
-  // last blocks, are dealt to the warps round-robin; a barrier ends the level.
+  const int nl = ctl[kCtlLevels];
+  const long long want = ctl[kCtlWant];
+  const int4* items = reinterpret_cast<const int4*>(ctl + kCtlItems);
+  bool direct = false;                                  // the root's blocks go straight out
+  if constexpr (LINEAR) {
+    const int4 root = *reinterpret_cast<const int4*>(ctl + kCtlLevel0 + 4 * nl);
+    direct = root.y == root.z && ((uintptr_t)dstg & 15u) == 0;
+  }
   for (int lv = 1; lv <= nl; ++lv) {
-    const unsigned lvm = __ballot_sync(0xffffffffu, is_node && c_level == lv);
-    const int n0 = __ffs(lvm) - 1, n1 = 31 - __clz(lvm);
-    const int it0 = __shfl_sync(0xffffffffu, c_first, n0);
-    const int it1 = __shfl_sync(0xffffffffu, c_end, n0);
-    const int big_end = __shfl_sync(0xffffffffu, c_first + c_nbig, n1);
+    const int4 info = *reinterpret_cast<const int4*>(ctl + kCtlLevel0 + 4 * lv);
     const KeyT* src = (lv & 1) ? bufX : bufY;           // level lv reads level lv-1's buffer
     KeyT* dst = (lv & 1) ? bufY : bufX;
-    for (int item = it0 + warp; item < it1; item += WARPS) {
-      int c, blk;
-      if (item < big_end) {                            // a big block: the node whose range holds it
-        const unsigned sel = __ballot_sync(0xffffffffu, is_node && c_first <= item && c_nbig > 0);
-        c = 31 - __clz(sel);
-        blk = item - __shfl_sync(0xffffffffu, c_first, c);
-      } else {                                         // a small block: its node's last
-        c = __ffs(__ballot_sync(0xffffffffu, is_node && c_small == item)) - 1;
-        blk = __shfl_sync(0xffffffffu, c_nb, c) - 1;
-      }
-      const int lenA = __shfl_sync(0xffffffffu, c_lenA, c);
-      const int lenB = __shfl_sync(0xffffffffu, c_lenB, c);
-      const int offA = __shfl_sync(0xffffffffu, c_offA, c);
-      const int offB = __shfl_sync(0xffffffffu, c_offB, c);
-      const int outo = __shfl_sync(0xffffffffu, c_out, c);
-      const KeyT* A = src + offA;
-      const KeyT* B = src + offB;
-      const int L = lenA + lenB;
-      const int d0 = blk * kBlockItems;
-      const int m = (L - d0) < kBlockItems ? (L - d0) : kBlockItems;
-      if (lenA != 0 && lenB != 0) {
-        int a0, a1;
-        block_coranks(A, lenA, B, lenB, d0, m, lane, a0, a1);
-        const int X = a1 - a0;
-        if (m <= kSmallBlockMax)
-          warp_merge_small<KeyT>(A + a0, X, B + (d0 - a0), m - X, dst + outo + d0, lane,
-                                 xout && lv == nl);
-        else
-          warp_merge_block<KeyT, MergeMix>(A + a0, X, B + (d0 - a0), m - X, dst + outo + d0, lane,
-                                 xout && lv == nl);
-      } else {
+    const bool xo = xout && lv == nl;
+    for (int at = info.x + warp; at < info.z; at += WARPS) {
+      const bool big = at < info.y;
+      const int4 it = items[at];
+      const int lenA = it.x >> 16, lenB = it.y >> 16, d0 = it.z >> 16, m = it.w;
+      const KeyT* A = src + (it.x & 0xFFFF);
+      const KeyT* B = src + (it.y & 0xFFFF);
+      KeyT* o = dst + (it.z & 0xFFFF) + d0;
+      if (!big && (lenA == 0 || lenB == 0)) {
         // One child is empty (a node over runs past the group's last, or a
         // tile that takes nothing from one side): the block is a copy, made
         // with 32 consecutive keys per access instead of a merge network.
         const KeyT* from = (lenB == 0 ? A : B) + d0;
-        KeyT* to = dst + outo + d0;
-        const bool xo = xout && lv == nl;
         for (int i = lane; i < m; i += 32) {
           const KeyT v = from[i];
-          to[i] = xo ? (KeyT)ordered_to_f32((uint32_t)v) : v;
+          o[i] = xo ? (KeyT)ordered_to_f32((uint32_t)v) : v;
+        }
+        __syncwarp();
+        continue;
+      }
+      int a0, a1;
+      block_coranks(A, lenA, B, lenB, d0, m, lane, a0, a1);
+      const int X = a1 - a0;
+      if (!big) {
+        warp_merge_small<KeyT>(A + a0, X, B + (d0 - a0), m - X, o, lane, xo);
+        __syncwarp();
+        continue;
+      }
+      if constexpr (!LINEAR) {
+        warp_merge_block<KeyT, MergeMix>(A + a0, X, B + (d0 - a0), m - X, o, lane, xo);
+        __syncwarp();
+        continue;
+      }
+      KeyT v[32];
+      warp_load_bitonic(A + a0, X, B + (d0 - a0), m - X, v, lane);
+      warp_bitonic_1024<MergeMix, false>(v, o, (m + 31) >> 5, lane);
+      const uint32_t ob = smem_u32addr(o), r = (uint32_t)lane & 7, g = (uint32_t)lane >> 3;
+      if (32 * lane < m) {
+#pragma unroll
+        for (int ch = 0; ch < 32 / E; ++ch) sts128(ob + lane * RB + ((ch ^ r) << 4), &v[ch * E]);
+      }
+      __syncwarp();
+#pragma unroll
+      for (int q = 0; q < 32 / E; ++q)                  // chunk 32q + lane: row 4q + g, place r
+        if (32 * E * q + E * lane < m)
+          lds_chunk(ob + (4 * q + g) * RB + ((r ^ g ^ (4 * (q & 1))) << 4), &v[q * E]);
+      if (xo) {
+#pragma unroll
+        for (int j = 0; j < 32; ++j) v[j] = (KeyT)ordered_to_f32((uint32_t)v[j]);
+      }
+      if (direct && lv == nl) {
+        KeyT* og = dstg + d0;
+#pragma unroll
+        for (int q = 0; q < 32 / E; ++q) {
+          const int pos = 32 * E * q + E * lane;
+          if (pos + E <= m)
+            *reinterpret_cast<typename Vec16<KeyT>::T*>(og + pos) = Vec16<KeyT>::pack(&v[q * E]);
+        }
+        if (m % E != 0) {                               // the chunk that straddles the end
+#pragma unroll
+          for (int q = 0; q < 32 / E; ++q) {
+            const int pos = 32 * E * q + E * lane;
+#pragma unroll
+            for (int w = 0; w < E - 1; ++w)
+              if (pos + w < m && pos + E > m) og[pos + w] = v[q * E + w];
+          }
+        }
+        continue;                                       // its item is the warp's last of the tile
+      }
+      __syncwarp();
+#pragma unroll
+      for (int q = 0; q < 32 / E; ++q)
+        sts128_if_le(ob + ((32 * q + lane) << 4), &v[q * E], 32 * E * q + E * lane + E, m);
+      if (m % E != 0) {
+#pragma unroll
+        for (int q = 0; q < 32 / E; ++q) {
+          const int pos = 32 * E * q + E * lane;
+#pragma unroll
+          for (int w = 0; w < E - 1; ++w)
+            if (pos + w < m && pos + E > m) sts_addr(ob + (uint32_t)((pos + w) * sizeof(KeyT)), v[q * E + w]);
         }
       }
       __syncwarp();
+    }
+    if (direct && lv == nl) {
+      fence_proxy_async_smem();                         // before a next tile's bulk copies
+      return;
     }
     sync();
   }
@@ -379,8 +454,8 @@ __device__ __forceinline__ void merge_levels(KeyT* bufX, KeyT* bufY, const int* 
 //      register-and-shuffle network of the smallest power of two that holds
 //      them (warp_merge_any); the last level, whose output is the whole block
 //      at its 16-byte aligned start, takes the transposed 1024-item network.
-// bufX holds the staged segments (the node table's level-1 entries give each
-// segment's span), bufY receives the tile; the final store is the same as the
+// bufX holds the staged segments (their offsets and lengths stand before the
+// pivot rows), bufY receives the tile; the final store is the same as the
 // tree's.
 // A warp whose pivot rows do not describe pieces inside their segments that
 // add up to its block records kDevErrInternal in dev_err and merges nothing,
@@ -391,22 +466,12 @@ __device__ __forceinline__ void merge_partition_blocks(const KeyT* bufX, KeyT* b
                                                        int* dev_err, Sync sync) {
   constexpr int E = Vec16<KeyT>::E;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int nl = ctl[kCtlNodeFields * 32 + 0];       // levels of the tree over the runs (>= 1)
-  const int want = ctl[kCtlNodeFields * 32 + 2];     // items of the tile
-  const int nnodes = ctl[kCtlNodeFields * 32 + 1];
+  const int nl = ctl[kCtlLevels];                    // levels of the tree over the runs (>= 1)
+  const int want = ctl[kCtlWant];                    // items of the tile
   const int nleaf = 1 << nl;                         // segments, empty past the group's runs
-  // Segment r is child A (r even) or B (r odd) of level-1 node r / 2; the
-  // node table lists nodes in level order, so only its level-1 entries give
-  // segments (with 5 runs, say, nodes 0..2 are level 1 and segments 6, 7 are
-  // empty).
-  int seg_off = 0, seg_len = 0;
-  {
-    const int q = lane >> 1;
-    if (lane < nleaf && q < nnodes && ctl[7 * 32 + q] == 1) {
-      seg_off = ctl[(2 + (lane & 1)) * 32 + q];
-      seg_len = ctl[(lane & 1) * 32 + q];
-    }
-  }
+  const int seg_off = lane < nleaf ? rows[lane] : 0;
+  const int seg_len = lane < nleaf ? rows[32 + lane] : 0;
+  rows += 64;
   const int nblk = (want + kBlockItems - 1) / kBlockItems;
   if (warp == 0) {
     rows[lane] = 0;
@@ -524,36 +589,41 @@ __device__ __forceinline__ bool merge_tile(const KeyT* __restrict__ in, KeyT* __
   const int cap = G::cap(K);
   KeyT* bufX = reinterpret_cast<KeyT*>(smem_raw);
   KeyT* bufY = bufX + cap;
-  int* ctl = reinterpret_cast<int*>(bar + 2);          // node table and scalars (see above)
+  int* ctl = reinterpret_cast<int*>(bar + 2);          // the control area (see above)
   // Every thread is past the previous tile (whose store has read its shared
   // memory) before the staging copies overwrite the buffer.
-  // Warp 0 stages the segments while warp 1 builds the node table.
+  // Warp 0 stages the segments while warp 1 lists the tree's blocks.
   long long lo = 0, hi = 0;
   if ((threadIdx.x >> 5) < 2)
     merge_tile_pivots(n, run_len, K, g, j, lo_row, hi_row, S, threadIdx.x & 31, lo, hi);
   __syncthreads();
+  // One thread polls the staging barrier; the others wait at the CTA barrier
+  // (no issue slots spent polling), which also orders the staged data, the
+  // plainly loaded items and the control area before every warp's reads.  The list is
+  // ready before the data is, so it costs the tile nothing.
+  bool ok = true;
   if ((threadIdx.x >> 5) < 2)
     merge_plan_warp<KeyT, WARPS>(in, n, run_len, K, g, j, lo, hi, S, bufX, ctl, bar,
-                                 threadIdx.x & 31, (threadIdx.x >> 5) == 0 ? 1 : 2);
-  __syncthreads();
-  if (ctl[kCtlNodeFields * 32 + 3] || (smem_u32addr(smem_raw) & 1023u) != 0) {
+                                 threadIdx.x & 31, (threadIdx.x >> 5) == 0 ? 1 : 2,
+                                 PARTITION ? ctl + kCtlInts : nullptr);
+  if (threadIdx.x == 0 && !ctl[kCtlErr]) {             // written by this thread
+    ok = mbar_wait_bounded(bar, phase);
+    if (test_timeout && ok) {
+      mbar_arrive_expect_tx(bar + 1, 16u);
+      ok = mbar_wait_bounded(bar + 1, 0u, 2000000ll);
+    }
+  }
+  const bool late = __syncthreads_or(!ok);
+  if (ctl[kCtlErr] || (smem_u32addr(smem_raw) & 1023u) != 0) {
     if (threadIdx.x == 0) set_device_error(dev_err, kDevErrInternal);
     return false;                                      // uniform over the CTA
   }
-  // One thread polls the staging barrier; the others wait at the CTA barrier
-  // (no issue slots spent polling), which also orders the staged data and the
-  // plainly loaded items before every warp's reads.
-  bool ok = (threadIdx.x == 0) ? mbar_wait_bounded(bar, phase) : true;
-  if (test_timeout && threadIdx.x == 0 && ok) {
-    mbar_arrive_expect_tx(bar + 1, 16u);
-    ok = mbar_wait_bounded(bar + 1, 0u, 2000000ll);
-  }
-  if (__syncthreads_or(!ok)) {
+  if (late) {
     if (threadIdx.x == 0) set_device_error(dev_err, kDevErrTimeout);
     return false;
   }
   if constexpr (PARTITION)
-    merge_partition_blocks<KeyT, WARPS>(bufX, bufY, ctl, ctl + kCtlNodeFields * 32 + kCtlScalars,
+    merge_partition_blocks<KeyT, WARPS>(bufX, bufY, ctl, ctl + kCtlInts,
                                         out + g * run_len * K + j * S, xout, dev_err,
                                         []() { __syncthreads(); });
   else

@@ -127,21 +127,18 @@ __device__ __forceinline__ void cas_dir(uint64_t& a, uint64_t& b, uint32_t f) {
 // multiply-add form gave 1.41x the compare-exchange rate of min/max alone
 // (10 of 16 for the per-lane-direction form, 1.38x).  Inside the kernels the
 // best mix follows what else the kernel issues, measured on GB300: the base
-// case (issue-bound, ALU pipe 69% busy) is fastest with 6 of 16 plain pairs
-// and 12 of 16 direction pairs, the merge pass (barrier-bound, ALU 57%) with
-// plain pairs as min/max and 12 of 16 direction pairs; each kernel passes its
-// own Mix type.  The multiply-adds use a runtime 1 (and -1, -2) so that the
+// case is fastest with 8 of 16 plain pairs (16.8 * 10^6 keys: 101 us, 107 with 4,
+// 110 with none) and 12 of 16 direction pairs, the merge pass with 6 plain pairs
+// (K = 16: 90.3 us, 92.3 with none, 92.5 with 8); each kernel passes its own Mix type.  The multiply-adds use a runtime 1 (and -1, -2) so that the
 // compiler keeps them multiplies.
 //
-// 64-bit keys: a compare-exchange is one 64-bit compare and four 32-bit
-// selects on the ALU pipe.  The selects can also be made exact multiply-adds
-// on the FMA pipe: with f = 1 when the pair swaps, each half x of a and y of
-// b becomes x + f (y - x) and y + f (x - y).  That form costs more issue
-// slots, so it pays only where the ALU pipe is the tighter limit: measured on
-// GB300 at 10^8 u64 keys, 6 of 16 plain pairs of the merge pass in it took the
-// five K = 8 passes from 4.686 to 4.594 ms, while any share of the base
-// case's pairs, or of direction pairs, made it slower (base case 1.85 ->
-// 2.00..2.30 ms).
+// 64-bit keys: a compare-exchange is one 64-bit compare (two instructions) and
+// four 32-bit selects on the ALU pipe.  In the other form two selects give the
+// lower key and the other key is what is left of the sums of the halves: four
+// ALU instructions and four on the FMA pipe.  Measured on GB300 at 2 * 10^7 u64 keys,
+// the base case is fastest with all its pairs in it (279 us with none, 271 with a
+// quarter, 262 with all), the merge pass, which waits for barriers and instructions
+// more than for a pipe, with none (K = 4: 125.4 us, 127.2 with 6 of 16, 131.5 with all).
 // ---------------------------------------------------------------------------
 // MIX / MIXD: how many of a stage's 16 pairs take the multiply-add form, for
 // plain pairs and for pairs whose direction is chosen per lane, with 32-bit
@@ -254,19 +251,23 @@ __device__ __forceinline__ uint32_t smem_u32addr(const void* p) {
 
 // Loads p[0] into v when idx < lim (signed), in one compare and one predicated
 // load; v keeps its value otherwise.
-__device__ __forceinline__ void lds_if_lt(uint32_t& v, const uint32_t* p, int idx, int lim) {
+__device__ __forceinline__ void lds_if_lt(uint32_t& v, uint32_t addr, int idx, int lim) {
   asm volatile(
       "{\n\t.reg .pred q;\n\tsetp.lt.s32 q, %2, %3;\n\t@q ld.shared.b32 %0, [%1];\n\t}\n"
       : "+r"(v)
-      : "r"(smem_u32addr(p)), "r"(idx), "r"(lim)
+      : "r"(addr), "r"(idx), "r"(lim)
       : "memory");
 }
-__device__ __forceinline__ void lds_if_lt(uint64_t& v, const uint64_t* p, int idx, int lim) {
+__device__ __forceinline__ void lds_if_lt(uint64_t& v, uint32_t addr, int idx, int lim) {
   asm volatile(
       "{\n\t.reg .pred q;\n\tsetp.lt.s32 q, %2, %3;\n\t@q ld.shared.b64 %0, [%1];\n\t}\n"
       : "+l"(v)
-      : "r"(smem_u32addr(p)), "r"(idx), "r"(lim)
+      : "r"(addr), "r"(idx), "r"(lim)
       : "memory");
+}
+template <typename KeyT>
+__device__ __forceinline__ void lds_if_lt(KeyT& v, const KeyT* p, int idx, int lim) {
+  lds_if_lt(v, smem_u32addr(p), idx, lim);
 }
 __device__ __forceinline__ uint32_t lds_key(const uint32_t* p) {
   uint32_t v;
@@ -299,19 +300,23 @@ __device__ __forceinline__ void lds_pair(uint64_t& v, const uint64_t* a, const u
       : "memory");
 }
 // Loads p[0] into v when idx >= lim (signed).
-__device__ __forceinline__ void lds_if_ge(uint32_t& v, const uint32_t* p, int idx, int lim) {
+__device__ __forceinline__ void lds_if_ge(uint32_t& v, uint32_t addr, int idx, int lim) {
   asm volatile(
       "{\n\t.reg .pred q;\n\tsetp.ge.s32 q, %2, %3;\n\t@q ld.shared.b32 %0, [%1];\n\t}\n"
       : "+r"(v)
-      : "r"(smem_u32addr(p)), "r"(idx), "r"(lim)
+      : "r"(addr), "r"(idx), "r"(lim)
       : "memory");
 }
-__device__ __forceinline__ void lds_if_ge(uint64_t& v, const uint64_t* p, int idx, int lim) {
+__device__ __forceinline__ void lds_if_ge(uint64_t& v, uint32_t addr, int idx, int lim) {
   asm volatile(
       "{\n\t.reg .pred q;\n\tsetp.ge.s32 q, %2, %3;\n\t@q ld.shared.b64 %0, [%1];\n\t}\n"
       : "+l"(v)
-      : "r"(smem_u32addr(p)), "r"(idx), "r"(lim)
+      : "r"(addr), "r"(idx), "r"(lim)
       : "memory");
+}
+template <typename KeyT>
+__device__ __forceinline__ void lds_if_ge(KeyT& v, const KeyT* p, int idx, int lim) {
+  lds_if_ge(v, smem_u32addr(p), idx, lim);
 }
 
 // ---------------------------------------------------------------------------
@@ -340,8 +345,8 @@ __device__ __forceinline__ int warp_corank(const KeyT* A, int lenA, const KeyT* 
   return lo;
 }
 
-// Both co-ranks of a full block, of d and of d + m, in one search: lanes 0-15
-// look for the first, lanes 16-31 for the second, each 16 probes a round (an odd
+// Both co-ranks of a block, of d and of d + m, in one search: lanes 0-15 look
+// for the first, lanes 16-31 for the second, each 16 probes a round (an odd
 // stride: at most two probes per bank).  Up to 4912 items in three rounds; one after
 // the other, 32 probes each, took five dependent rounds (the second search
 // bracketed by the first).
@@ -519,46 +524,55 @@ __device__ __forceinline__ void load_chunk(uint32_t addr, uint64_t* v) {
   v[2] = ((uint64_t)y.z << 32) | x.z; v[3] = ((uint64_t)y.w << 32) | x.w;
 }
 
-// Striped -> blocked through `out` (16-byte aligned, 32 * nr items).  Row k
-// takes the k-th 128 bytes (8-byte keys: 128 bytes of low halves, then 128 of
-// high halves) with its eight 16-byte chunks XOR-swizzled by k & 7, so the row
-// stores (stmatrix; a last group of fewer than four rows word by word) and
-// the 16-byte row loads are both conflict-free.  Rows at or above nr are not
-// stored; lanes at or above nr receive pads.
+// Striped -> blocked goes through shared memory: row k takes 128 bytes (8-byte
+// keys: 128 bytes of low halves, then 128 of high halves) with its eight 16-byte
+// chunks XOR-swizzled by k & 7, so the row stores (stmatrix; rows of a group of four
+// that are not all wanted word by word) and the 16-byte row loads are both
+// conflict-free.
+
+// Stores rows 4q .. 4q + 3 of which nr are wanted (nr >= 4: all) at ob, the first of them; 4q
+// counts from a row whose swizzle is 0.
 template <typename KeyT>
-__device__ __forceinline__ void striped_to_blocked(KeyT (&v)[32], KeyT* out, int nr, int lane) {
+__device__ __forceinline__ void store_striped4(const KeyT* v, uint32_t ob, int q, int nr, int lane) {
   constexpr uint32_t RB = 32 * sizeof(KeyT);
-  const uint32_t ob = smem_u32addr(out);
   const uint32_t i = (uint32_t)lane >> 3, r = (uint32_t)lane & 7;
-  const uint32_t a0 = ob + i * RB + ((r ^ i) << 4);           // rows 8p + i
-  const uint32_t a1 = ob + i * RB + ((r ^ i ^ 4) << 4);       // rows 8p + 4 + i
-  const uint32_t row = ob + (uint32_t)lane * RB;
-  if (nr == 32) {
+  if (nr >= 4) {
+    store_rows4(ob + i * RB + ((r ^ i ^ (4 * (q & 1))) << 4), v);
+  } else {
 #pragma unroll
-    for (int q = 0; q < 8; ++q) store_rows4(((q & 1) ? a1 : a0) + 4 * q * RB, &v[4 * q]);
-    __syncwarp();
+    for (int k = 0; k < 4; ++k)
+      if (k < nr) store_word(ob + k * RB + (((uint32_t)lane ^ (4 * (k + 4 * (q & 1)))) << 2), v[k]);
+  }
+}
+
+// The lane's row from shared address `row`; pads where it is not live.
+template <typename KeyT>
+__device__ __forceinline__ void load_row(KeyT (&v)[32], uint32_t row, bool live, int lane) {
+  const uint32_t r = (uint32_t)lane & 7;
+  if (live) {
 #pragma unroll
     for (int ch = 0; ch < 8; ++ch) load_chunk(row + ((ch ^ r) << 4), &v[4 * ch]);
   } else {
 #pragma unroll
-    for (int q = 0; q < 8; ++q) {
-      if (4 * q + 3 < nr) {
-        store_rows4(((q & 1) ? a1 : a0) + 4 * q * RB, &v[4 * q]);
-      } else {
-#pragma unroll
-        for (int k = 4 * q; k < 4 * q + 4; ++k)
-          if (k < nr) store_word(ob + k * RB + (((uint32_t)lane ^ (4 * (k & 7))) << 2), v[k]);
-      }
-    }
-    __syncwarp();
-    if (lane < nr) {
-#pragma unroll
-      for (int ch = 0; ch < 8; ++ch) load_chunk(row + ((ch ^ r) << 4), &v[4 * ch]);
-    } else {
-#pragma unroll
-      for (int k = 0; k < 32; ++k) v[k] = key_pad<KeyT>();
-    }
+    for (int k = 0; k < 32; ++k) v[k] = key_pad<KeyT>();
   }
+}
+
+// Striped -> blocked through `out` (16-byte aligned, 32 * nr items).  Rows at or
+// above nr are not stored; lanes at or above nr receive pads.
+template <typename KeyT>
+__device__ __forceinline__ void striped_to_blocked(KeyT (&v)[32], KeyT* out, int nr, int lane) {
+  constexpr uint32_t RB = 32 * sizeof(KeyT);
+  const uint32_t ob = smem_u32addr(out);
+  if (nr == 32) {
+#pragma unroll
+    for (int q = 0; q < 8; ++q) store_striped4(&v[4 * q], ob + 4 * q * RB, q, 4, lane);
+  } else {
+#pragma unroll
+    for (int q = 0; q < 8; ++q) store_striped4(&v[4 * q], ob + 4 * q * RB, q, nr - 4 * q, lane);
+  }
+  __syncwarp();
+  load_row(v, ob + (uint32_t)lane * RB, lane < nr, lane);
   __syncwarp();
 }
 
@@ -593,7 +607,8 @@ __device__ __forceinline__ void blocked_stages(KeyT (&v)[32], int lane, const M&
 // (every item of row k is <= every item of row k+1), so rows at or above
 // nr = ceil(m / 32) hold only pads (or real all-ones keys, bit-identical to
 // pads) and are neither stored nor loaded.  M: the kernel's compare-exchange mix.
-template <typename M, typename KeyT>
+// FLIP: end in warp_store_block's layout.
+template <typename M, bool FLIP = true, typename KeyT>
 __device__ __forceinline__ void warp_bitonic_1024(KeyT (&v)[32], KeyT* out, int nr, int lane) {
   const M c = mad_ones<M>();
   striped_stage<16>(v, c);                           // strides 512 .. 32
@@ -602,7 +617,7 @@ __device__ __forceinline__ void warp_bitonic_1024(KeyT (&v)[32], KeyT* out, int 
   striped_stage<2>(v, c);
   striped_stage<1>(v, c);
   striped_to_blocked(v, out, nr, lane);
-  blocked_stages<true>(v, lane, c);                  // strides 16 .. 1, store layout
+  blocked_stages<FLIP>(v, lane, c);                  // strides 16 .. 1
 }
 __device__ __forceinline__ void sts_addr(uint32_t addr, uint32_t v) {
   asm volatile("st.shared.b32 [%0], %1;" ::"r"(addr), "r"(v) : "memory");
@@ -657,15 +672,15 @@ __device__ __forceinline__ void sts128_if_le(uint32_t addr, const uint64_t* v, i
       : "memory");
 }
 
-// Stores the sorted block: register j of the lane holds item 32*lane + (j ^ F),
-// F = flip_mask(lane).  `out` must be 16-byte aligned.  Items go out in 16-byte
-// chunks (chunk c of the lane lands at chunk c ^ (F / E) of its row); for a
-// short block the chunks wholly below m are stored this way and the one chunk
-// that straddles m item by item (by a single lane).  `xout` undoes the float
+// Stores the lane's row of a sorted block: register j holds item j ^ F of the
+// row, F = flip_mask(lane), and `room` of the row's 32 items lie in the block
+// (32 or more: all).  `row`: the row's 16-byte aligned shared address.  Items
+// go out in 16-byte chunks (chunk c lands at chunk c ^ (F / E) of the row); the one chunk that
+// straddles the block's end goes item by item.  `xout` undoes the float
 // transform on the way out.
 template <typename KeyT>
-__device__ __forceinline__ void warp_store_block(KeyT* out, int m, KeyT (&v)[32], int lane,
-                                                 bool xout) {
+__device__ __forceinline__ void warp_store_row(uint32_t row, int room, bool full, KeyT (&v)[32],
+                                               int lane, bool xout) {
   constexpr int E = Vec16<KeyT>::E;
   constexpr int SZ = (int)sizeof(KeyT);
   if (xout) {
@@ -673,14 +688,12 @@ __device__ __forceinline__ void warp_store_block(KeyT* out, int m, KeyT (&v)[32]
     for (int j = 0; j < 32; ++j) v[j] = (KeyT)ordered_to_f32((uint32_t)v[j]);
   }
   const int F = flip_mask<KeyT>(lane);
-  const uint32_t row = smem_u32addr(out + 32 * lane);
-  const int room = m - 32 * lane;                    // items of this row below m
 #pragma unroll
   for (int c = 0; c < 32 / E; ++c) {
     const int pos = (c * E) ^ F;                      // item offset of the chunk in the row
     sts128_if_le(row + (uint32_t)(pos * SZ), &v[c * E], pos + E, room);
   }
-  if (m < kBlockItems && (m % E) != 0) {
+  if (!full) {
 #pragma unroll
     for (int c = 0; c < 32 / E; ++c) {
       const int pos = (c * E) ^ F;
@@ -690,6 +703,14 @@ __device__ __forceinline__ void warp_store_block(KeyT* out, int m, KeyT (&v)[32]
           sts_addr(row + (uint32_t)((pos + w) * SZ), v[c * E + w]);
     }
   }
+}
+
+// Stores the sorted block of m items in the blocked layout above to out (16-byte aligned).
+template <typename KeyT>
+__device__ __forceinline__ void warp_store_block(KeyT* out, int m, KeyT (&v)[32], int lane,
+                                                 bool xout) {
+  warp_store_row<KeyT>(smem_u32addr(out + 32 * lane), m - 32 * lane,
+                       m == kBlockItems || m % Vec16<KeyT>::E == 0, v, lane, xout);
 }
 
 // `out` is 16-byte aligned; the warp may use out[0, 32 * ceil((X + Y) / 32))
@@ -751,7 +772,7 @@ __device__ __forceinline__ void warp_merge_small_r(const KeyT* A, int X, const K
 #pragma unroll
     for (int k = 0; k < R; ++k) {
       const KeyT y = __shfl_xor_sync(0xffffffffu, v[k], s);
-      v[k] = upper ? kmax(v[k], y) : kmin(v[k], y);
+      v[k] = (y < v[k]) != upper ? y : v[k];
     }
   }
 #pragma unroll
@@ -767,10 +788,15 @@ template <typename KeyT>
 __device__ __forceinline__ void warp_merge_small(const KeyT* A, int X, const KeyT* B, int Y,
                                                  KeyT* out, int lane, bool xout) {
   const int m = X + Y;
-  if (m <= 32) warp_merge_small_r<1>(A, X, B, Y, out, lane, xout);
-  else if (m <= 64) warp_merge_small_r<2>(A, X, B, Y, out, lane, xout);
-  else if (m <= 128) warp_merge_small_r<4>(A, X, B, Y, out, lane, xout);
-  else warp_merge_small_r<8>(A, X, B, Y, out, lane, xout);
+  if constexpr (sizeof(KeyT) == 8) {                 // fewer sizes: 8-byte kernels wait for instructions
+    if (m <= 64) warp_merge_small_r<2>(A, X, B, Y, out, lane, xout);
+    else warp_merge_small_r<8>(A, X, B, Y, out, lane, xout);
+  } else {
+    if (m <= 32) warp_merge_small_r<1>(A, X, B, Y, out, lane, xout);
+    else if (m <= 64) warp_merge_small_r<2>(A, X, B, Y, out, lane, xout);
+    else if (m <= 128) warp_merge_small_r<4>(A, X, B, Y, out, lane, xout);
+    else warp_merge_small_r<8>(A, X, B, Y, out, lane, xout);
+  }
 }
 
 // Merges A[0, X) and B[0, Y) (X + Y <= 1024, any shared-memory offsets) into

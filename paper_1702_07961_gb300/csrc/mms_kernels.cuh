@@ -17,10 +17,10 @@ constexpr int kMaxFanout = 32;
 // min and two multiply-adds instead of min and max, per kernel: the base
 // case and the merge pass (plain pairs, pairs with a per-lane direction).
 constexpr int kTileMadPairs = 8, kTileMadDirPairs = 12;
-constexpr int kMergeMadPairs = 0, kMergeMadDirPairs = 12;
+constexpr int kMergeMadPairs = 6, kMergeMadDirPairs = 12;
 // The same for 64-bit keys (their selects as multiply-adds; see mms_common.cuh).
 constexpr int kTileMad64Pairs = 16, kTileMad64DirPairs = 0;
-constexpr int kMergeMad64Pairs = 6, kMergeMad64DirPairs = 0;
+constexpr int kMergeMad64Pairs = 0, kMergeMad64DirPairs = 0;
 
 // Device error word values (the first word of a sort workspace).
 constexpr int kDevOk = 0;
