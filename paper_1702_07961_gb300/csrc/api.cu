@@ -213,15 +213,10 @@ __global__ void forward_status_kernel(const int* __restrict__ ws_status) {
   if (w != 0) atomicCAS(&g_stream_status, 0, w);
 }
 
-// Allocates a workspace stream-ordered and clears its status word.
+// Allocates a workspace stream-ordered.
 mms_status alloc_workspace(void** d_ws, size_t bytes, cudaStream_t s) {
-  cudaError_t e = cudaMallocAsync(d_ws, bytes, s);
+  const cudaError_t e = cudaMallocAsync(d_ws, bytes, s);
   if (e != cudaSuccess) return fail(MMS_ERR_NO_MEMORY, "cudaMallocAsync of the workspace failed%s");
-  e = cudaMemsetAsync(*d_ws, 0, kStatusBytes, s);
-  if (e != cudaSuccess) {
-    cudaFreeAsync(*d_ws, s);
-    return cuda_fail(e, "workspace init");
-  }
   return MMS_OK;
 }
 
@@ -237,8 +232,8 @@ mms_status release_workspace(void* d_ws, cudaStream_t s, mms_status st) {
   return st;
 }
 
-// Clears the status word of a caller's workspace on the stream, so that a
-// stale or uninitialised word never reads as this call's error.
+// Clears a workspace's status word on the stream, so that a stale or uninitialised
+// word never reads as this call's error, where the sort's first kernel does not.
 mms_status clear_status(void* d_ws, cudaStream_t s) {
   const cudaError_t e = cudaMemsetAsync(d_ws, 0, sizeof(int), s);
   return e == cudaSuccess ? MMS_OK : cuda_fail(e, "status word");
@@ -360,25 +355,29 @@ mms_status mms_sort_keys_ex(mms_key_type kt, void* d_keys, size_t n, void* d_ws,
     return fail(MMS_ERR_INVALID_ARG, "the partition and pipelined merge variants take the default tile geometry (tile_items and merge_tile_items 0) and no test flags%s");
   const WsLayout L = ws_layout(kt, n, 0);
   cudaStream_t s = (cudaStream_t)stream;
+  int K[64];
+  const int rounds = plan_rounds(kb, n, opt, K, 64);
+  long long run_len = base_run_items(kb, n, opt);      // of the base case
+  const bool cluster = run_len != S;
   bool owned = false;
   if (d_ws) {
     if (!aligned16(d_ws)) return fail(MMS_ERR_INVALID_ARG, "workspace not 16-byte aligned%s");
     if (ws_bytes < L.total) return fail(MMS_ERR_NO_MEMORY, "workspace smaller than mms_sort_workspace_bytes()%s");
-    const mms_status cs = clear_status(d_ws, s);
-    if (cs != MMS_OK) return cs;
-  } else {
+  } else if (rounds > 0) {                              // one base-case run is sorted in place, without one
     const mms_status as = alloc_workspace(&d_ws, L.total, s);
     if (as != MMS_OK) return as;
     owned = true;
   }
+  if (d_ws && cluster) {                                // else the base case clears it
+    const mms_status cs = clear_status(d_ws, s);
+    if (cs != MMS_OK) return owned ? release_workspace(d_ws, s, cs) : cs;
+  }
   unsigned char* ws = static_cast<unsigned char*>(d_ws);
   int* dev_err = reinterpret_cast<int*>(ws);
   const bool test_timeout = opt && (opt->test_flags & MMS_TEST_STAGING_TIMEOUT);
-  void* tmp = ws + L.keys_off;
-  long long* table = reinterpret_cast<long long*>(ws + L.table_off);
+  void* tmp = ws ? ws + L.keys_off : nullptr;
+  long long* table = ws ? reinterpret_cast<long long*>(ws + L.table_off) : nullptr;
 
-  int K[64];
-  const int rounds = plan_rounds(kb, n, opt, K, 64);
   const bool is_f32 = kt == MMS_KEY_F32;
   mms_status st = MMS_OK;
   // Base case writes to the caller's buffer when an even number of rounds follows.
@@ -393,10 +392,9 @@ mms_status mms_sort_keys_ex(mms_key_type kt, void* d_keys, size_t n, void* d_ws,
   mark();
   // The base case: one CTA per tile, or one thread-block cluster per run of
   // several tiles.
-  long long run_len = base_run_items(kb, n, opt);
-  st = check_launch(run_len == S
+  st = check_launch(!cluster
                         ? mms::launch_tile_sort(kb, tw, is_f32, is_f32 && rounds == 0, d_keys, cur,
-                                                (long long)n, s)
+                                                (long long)n, dev_err, s)
                         : mms::launch_tile_sort_cluster((int)(run_len / S), is_f32,
                                                         is_f32 && rounds == 0, d_keys, cur,
                                                         (long long)n, s),
@@ -435,7 +433,7 @@ mms_status mms_sort_keys(mms_key_type kt, void* d_keys, size_t n, void* d_ws, si
 // are copied first, so d_keys / d_values are overwritten only by the last
 // kernel): composite base case, merge rounds, key write-back and value gather.
 static mms_status pairs32_run(bool is_f32, void* d_keys, uint32_t* d_values, size_t n,
-                              unsigned char* ws, const WsLayout& L, cudaStream_t s,
+                              unsigned char* ws, const WsLayout& L, bool clear, cudaStream_t s,
                               const mms_options* opt, int& ev) {
   int* dev_err = reinterpret_cast<int*>(ws);
   void* comp[2] = {ws + L.comp0_off, ws + L.comp1_off};
@@ -462,7 +460,8 @@ static mms_status pairs32_run(bool is_f32, void* d_keys, uint32_t* d_values, siz
   cudaError_t ce = cudaMemcpyAsync(vcopy, d_values, n * sizeof(uint32_t), cudaMemcpyDeviceToDevice, s);
   if (ce != cudaSuccess) st = cuda_fail(ce, "copy of the values");
   if (st == MMS_OK)
-    st = check_launch(mms::launch_tile_sort_composite(tw, is_f32, d_keys, comp[0], (long long)n, s),
+    st = check_launch(mms::launch_tile_sort_composite(tw, is_f32, d_keys, comp[0], (long long)n,
+                                                      clear ? dev_err : nullptr, s),
                       "tile_sort (key-value)");
   mark();
   long long run_len = S;
@@ -518,19 +517,16 @@ mms_status mms_sort_pairs_ex(mms_key_type kt, void* d_keys, uint32_t* d_values, 
   if (d_ws) {
     if (!aligned16(d_ws)) return fail(MMS_ERR_INVALID_ARG, "workspace not 16-byte aligned%s");
     if (ws_bytes < L.total) return fail(MMS_ERR_NO_MEMORY, "workspace smaller than mms_sort_workspace_bytes()%s");
-    const mms_status cs = clear_status(d_ws, s);
-    if (cs != MMS_OK) return cs;
   } else {
     const mms_status as = alloc_workspace(&d_ws, L.total, s);
     if (as != MMS_OK) return as;
     owned = true;
   }
   unsigned char* ws = static_cast<unsigned char*>(d_ws);
-  int* dev_err = reinterpret_cast<int*>(ws);
   int ev = 0;
   mms_status st = MMS_OK;
   if (kt != MMS_KEY_U64) {
-    st = pairs32_run(kt == MMS_KEY_F32, d_keys, d_values, n, ws, L, s, opt, ev);
+    st = pairs32_run(kt == MMS_KEY_F32, d_keys, d_values, n, ws, L, true, s, opt, ev);
   } else {
     // Two stable 4-byte passes, low half first (see pairs.cu).
     void* half = ws + L.half_off;
@@ -540,12 +536,12 @@ mms_status mms_sort_pairs_ex(mms_key_type kt, void* d_keys, uint32_t* d_values, 
     st = check_launch(mms::launch_u64_pairs_split(d_keys, d_values, half, perm, kcopy, vcopy,
                                                   (long long)n, s), "key-value split (8-byte keys)");
     if (st == MMS_OK)
-      st = pairs32_run(false, half, static_cast<uint32_t*>(perm), n, ws, L, s, opt, ev);
+      st = pairs32_run(false, half, static_cast<uint32_t*>(perm), n, ws, L, true, s, opt, ev);
     if (st == MMS_OK)
       st = check_launch(mms::launch_u64_pairs_hi(kcopy, perm, half, (long long)n, s),
                         "key-value high halves (8-byte keys)");
     if (st == MMS_OK)
-      st = pairs32_run(false, half, static_cast<uint32_t*>(perm), n, ws, L, s, opt, ev);
+      st = pairs32_run(false, half, static_cast<uint32_t*>(perm), n, ws, L, false, s, opt, ev);
     if (st == MMS_OK)
       st = check_launch(mms::launch_u64_pairs_final(kcopy, vcopy, perm, d_keys, d_values,
                                                     (long long)n, s),
@@ -568,7 +564,7 @@ mms_status mms_tile_sort(mms_key_type kt, const void* d_in, void* d_out, size_t 
     return fail(MMS_ERR_INVALID_ARG, "buffers null or not aligned to the key size%s");
   const bool f = kt == MMS_KEY_F32;
   return check_launch(mms::launch_tile_sort(kb, mms::default_tile_warps(kb), f, f, d_in, d_out, (long long)n,
-                                            (cudaStream_t)stream), "tile_sort");
+                                            nullptr, (cudaStream_t)stream), "tile_sort");
 }
 
 size_t mms_splitter_rows(mms_key_type kt, size_t n, size_t run_len, int K) {

@@ -64,8 +64,10 @@ size_t merge_pass_smem_bytes(int key_bytes, int warps, int K);
 
 // Base case: sorts every tile of 1024 * tile_warps keys; in == out allowed.
 // xin / xout: apply the float order transform on load / its inverse on store.
+// status: a status word to clear, or nullptr.  Launched with programmatic
+// stream serialization behind whatever is on the stream.
 cudaError_t launch_tile_sort(int key_bytes, int tile_warps, bool xin, bool xout, const void* in,
-                             void* out, long long n, cudaStream_t s);
+                             void* out, long long n, int* status, cudaStream_t s);
 
 // Base case over runs of cluster_ctas * 8192 4-byte keys (cluster_ctas 2, 4
 // or 8): one thread-block cluster per run, each CTA sorting one 8192-key tile,
@@ -77,7 +79,7 @@ cudaError_t launch_tile_sort_cluster(int cluster_ctas, bool xin, bool xout, cons
 // Base case of the key-value sort: 32-bit keys -> sorted tiles of 64-bit
 // composites (ordered key << 32 | array position).
 cudaError_t launch_tile_sort_composite(int tile_warps, bool xin, const void* keys32, void* out64,
-                                       long long n, cudaStream_t s);
+                                       long long n, int* status, cudaStream_t s);
 
 // Last step of the key-value sort: keys back from the sorted composites, and
 // each value gathered from its original position.
