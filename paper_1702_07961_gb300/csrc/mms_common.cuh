@@ -242,6 +242,14 @@ using TileMix = Mix<kTileMadPairs, kTileMadDirPairs, kTileMad64Pairs, kTileMad64
 using MergeMix = Mix<kMergeMadPairs, kMergeMadDirPairs, kMergeMad64Pairs, kMergeMad64DirPairs>;
 
 
+// The warp's index, known to the compiler to be uniform (a shuffle's result from
+// one lane is): a branch on it needs no reconvergence code, and no warp
+// synchronisation around the collectives inside.  Without it the branch of
+// tile_idle_warp made the tile sort 12% slower.
+__device__ __forceinline__ int warp_index() {
+  return __shfl_sync(0xffffffffu, (int)(threadIdx.x >> 5), 0);
+}
+
 // ---------------------------------------------------------------------------
 // Shared-memory accesses the compiler may not merge or reorder across.
 // ---------------------------------------------------------------------------

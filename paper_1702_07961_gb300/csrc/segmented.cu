@@ -81,18 +81,28 @@ __device__ __forceinline__ Desc load_desc(const Desc* d) {
 }
 
 // ---- planner --------------------------------------------------------------
+//
+// Three kernels of 4 to 6 us each; like the base case and the merge rounds after them
+// they are launched with programmatic serialization, so that one starts where
+// the one before it ends.  The scan clears the status word, or records a fault the
+// plan marked (a memset before the plan was a launch more).
+
+constexpr int kBadSegment = 1 << 8;               // in segK: offsets or size out of bounds
 
 // One thread per segment: K, R and the tile count of every phase.
 __global__ void seg_plan_kernel(const unsigned long long* __restrict__ off, long long nseg,
                                 unsigned long long total_n, SegPlan P, int* __restrict__ segK,
-                                int* __restrict__ segR, int* __restrict__ counts, int* dev_err) {
+                                int* __restrict__ segR, int* __restrict__ counts) {
+  griddep_wait();
+  griddep_launch_dependents();
   const long long s = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (s >= nseg) return;
+  int bad = 0;
   const unsigned long long a = off[s], b = off[s + 1];
   long long n = 0;
   if (b < a || b > total_n || (s == 0 && a != 0) || (s == nseg - 1 && b != total_n) ||
       b - a > 0xFFFFFFFFull) {
-    set_device_error(dev_err, kDevErrInternal);   // offsets out of order or too large
+    bad = kBadSegment;                            // offsets out of order or too large
   } else {
     n = (long long)(b - a);
   }
@@ -101,10 +111,10 @@ __global__ void seg_plan_kernel(const unsigned long long* __restrict__ off, long
   K = K < 2 ? 2 : (K > P.kmax ? P.kmax : K);
   int R = rounds_for(tiles, K);
   if (R > P.rounds) {
-    set_device_error(dev_err, kDevErrInternal);   // a segment above the declared maximum
+    bad = kBadSegment;                            // a segment above the declared maximum
     R = P.rounds;
   }
-  segK[s] = K;
+  segK[s] = K | bad;
   segR[s] = R;
   counts[s] = (int)tiles;                         // phase 0: base case
   long long run_len = P.S;
@@ -115,11 +125,25 @@ __global__ void seg_plan_kernel(const unsigned long long* __restrict__ off, long
 }
 
 // One CTA per phase: exclusive scan of the phase's counts in place, total
-// into totals[phase].
+// into totals[phase].  Phase 0's CTA also sets the status word: to an error when a
+// segment is marked bad, else to 0 (`clear`) or not at all.
 __global__ void __launch_bounds__(1024) seg_scan_kernel(int* __restrict__ counts, long long nseg,
-                                                        int* __restrict__ totals) {
+                                                        int* __restrict__ totals,
+                                                        const int* __restrict__ segK, int* dev_err,
+                                                        int clear) {
   __shared__ int warp_sums[32];
   __shared__ int carry_s;
+  griddep_wait();
+  griddep_launch_dependents();
+  if (blockIdx.x == 0) {
+    int bad = 0;
+    for (long long i = threadIdx.x; i < nseg; i += 1024) bad |= segK[i] & kBadSegment;
+    bad = __syncthreads_or(bad);
+    if (threadIdx.x == 0) {
+      if (clear) *dev_err = bad ? kDevErrInternal : kDevOk;
+      else if (bad) set_device_error(dev_err, kDevErrInternal);
+    }
+  }
   int* c = counts + (long long)blockIdx.x * nseg;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   if (threadIdx.x == 0) carry_s = 0;
@@ -161,6 +185,8 @@ __global__ void seg_desc_kernel(const unsigned long long* __restrict__ off, long
                                 const int* __restrict__ segK, const int* __restrict__ segR,
                                 const int* __restrict__ offs, const int* __restrict__ totals,
                                 long long per_phase, Desc* __restrict__ desc) {
+  griddep_wait();
+  griddep_launch_dependents();
   const int p = blockIdx.y;
   const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   // Offsets that overlap (flagged by the planner) can make the counts exceed
@@ -173,7 +199,7 @@ __global__ void seg_desc_kernel(const unsigned long long* __restrict__ off, long
     if (o[mid] <= t) lo = mid; else hi = mid - 1;
   }
   const long long s = lo;
-  const int K = segK[s], R = segR[s];
+  const int K = segK[s] & (kBadSegment - 1), R = segR[s];
   const unsigned idx = (unsigned)(t - o[s]);
   unsigned flip, last;
   if (p == 0) {
@@ -200,12 +226,14 @@ __global__ void __launch_bounds__(WARPS * 32, (TileMinBlocks<KeyT, WARPS>::value
                          long long per_phase) {
   extern __shared__ __align__(1024) unsigned char smem_raw[];
   constexpr int T = WARPS * kBlockItems;
+  griddep_wait();
+  griddep_launch_dependents();
   const int cnt = (int)min((long long)*total, per_phase);
   for (int t = blockIdx.x; t < cnt; t += gridDim.x) {
     const Desc d = load_desc(desc + t);
     const unsigned idx = d.w & 0x1FFFFFu;
     KeyT* out = ((d.w >> 27) & 1u) ? bufB : bufA;
-    tile_sort_tile<KeyT, WARPS, XIN>(keys_in + d.base, out + d.base, (long long)d.n,
+    tile_sort_tile<KeyT, WARPS, XIN, true>(keys_in + d.base, out + d.base, (long long)d.n,
                                      (long long)idx * T, XIN && ((d.w >> 28) & 1u), smem_raw);
   }
 }
@@ -217,12 +245,14 @@ __global__ void __launch_bounds__(WARPS * 32, (TileMinBlocks<uint64_t, WARPS>::v
                                    const int* __restrict__ total, long long per_phase) {
   extern __shared__ __align__(1024) unsigned char smem_raw[];
   constexpr int T = WARPS * kBlockItems;
+  griddep_wait();
+  griddep_launch_dependents();
   const int cnt = (int)min((long long)*total, per_phase);
   for (int t = blockIdx.x; t < cnt; t += gridDim.x) {
     const Desc d = load_desc(desc + t);
     const unsigned idx = d.w & 0x1FFFFFu;
     uint64_t* out = ((d.w >> 27) & 1u) ? bufB : bufA;
-    tile_sort_composite_tile<WARPS, XIN>(keys_in + d.base, out + d.base, (long long)d.n,
+    tile_sort_composite_tile<WARPS, XIN, true>(keys_in + d.base, out + d.base, (long long)d.n,
                                          (long long)idx * T, (long long)d.base, smem_raw);
   }
 }
@@ -272,6 +302,8 @@ __global__ void __launch_bounds__(WARPS * 32, (MinBlocks<KeyT, WARPS>::value))
   constexpr int S = WARPS * kBlockItems;
   uint64_t* bar = reinterpret_cast<uint64_t*>(smem_raw + bar_off);
   if (threadIdx.x == 0) mbar_init(bar, 1);
+  griddep_wait();                                 // the pivot table and the runs
+  griddep_launch_dependents();
   const int cnt = (int)min((long long)*total, per_phase);
   unsigned phase = 0;
   for (int t = blockIdx.x; t < cnt; t += gridDim.x) {
@@ -438,9 +470,8 @@ cudaError_t launch_seg_tile(const void* keys_in, void* a, void* b, const Desc* d
   unsigned grid = 1;
   if (e == cudaSuccess) e = persistent_grid(k, WARPS * 32, smem, upper, &grid);
   if (e != cudaSuccess) return e;
-  k<<<grid, WARPS * 32, smem, s>>>(static_cast<const KeyT*>(keys_in), static_cast<KeyT*>(a),
-                                   static_cast<KeyT*>(b), desc, total, upper);
-  return cudaGetLastError();
+  return launch_k(k, dim3(grid), dim3(WARPS * 32), smem, s, true, static_cast<const KeyT*>(keys_in),
+                  static_cast<KeyT*>(a), static_cast<KeyT*>(b), desc, total, upper);
 }
 
 template <int WARPS, bool XIN>
@@ -452,10 +483,10 @@ cudaError_t launch_seg_tile_comp(const void* keys_in, void* a, void* b, const De
   unsigned grid = 1;
   if (e == cudaSuccess) e = persistent_grid(k, WARPS * 32, smem, upper, &grid);
   if (e != cudaSuccess) return e;
-  k<<<grid, WARPS * 32, smem, s>>>(static_cast<const uint32_t*>(keys_in),
-                                   static_cast<uint64_t*>(a), static_cast<uint64_t*>(b), desc,
-                                   total, upper);
-  return cudaGetLastError();
+  // The value copy lies between this and the planner: the launch takes no early start then.
+  return launch_k(k, dim3(grid), dim3(WARPS * 32), smem, s, true,
+                  static_cast<const uint32_t*>(keys_in), static_cast<uint64_t*>(a),
+                  static_cast<uint64_t*>(b), desc, total, upper);
 }
 
 template <typename KeyT, int K2MAX, typename Idx>
@@ -497,9 +528,8 @@ cudaError_t launch_seg_merge(void* a, void* b, const Desc* desc, const int* tota
   unsigned grid = 1;
   if (e == cudaSuccess) e = persistent_grid(k, WARPS * 32, smem, upper, &grid);
   if (e != cudaSuccess) return e;
-  k<<<grid, WARPS * 32, smem, s>>>(static_cast<KeyT*>(a), static_cast<KeyT*>(b), desc, total,
-                                   upper, r, is_f32, table, bar_off, dev_err);
-  return cudaGetLastError();
+  return launch_k(k, dim3(grid), dim3(WARPS * 32), smem, s, true, static_cast<KeyT*>(a),
+                  static_cast<KeyT*>(b), desc, total, upper, r, is_f32, table, bar_off, dev_err);
 }
 
 cudaError_t seg_tile_phase(mms_key_type kt, bool pairs, int tw, const void* keys, void* a,
@@ -710,22 +740,19 @@ static mms_status seg_sort_impl(mms_key_type kt, void* d_keys, uint32_t* d_value
     return MMS_ERR_CUDA;
   };
   mark();
-  mms_status st = clear_status ? chk(cudaMemsetAsync(dev_err, 0, sizeof(int), s), "status word")
-                               : MMS_OK;
-  if (st == MMS_OK) {
-    seg_plan_kernel<<<(unsigned)((nseg + 255) / 256), 256, 0, s>>>(off, nseg, total_n, P, segK, segR,
-                                                                  counts, dev_err);
-    st = chk(cudaGetLastError(), "seg_plan");
-  }
-  if (st == MMS_OK) {
-    seg_scan_kernel<<<(unsigned)P.nphase, 1024, 0, s>>>(counts, nseg, totals);
-    st = chk(cudaGetLastError(), "seg_scan");
-  }
-  if (st == MMS_OK) {
-    dim3 g((unsigned)((L.per_phase + 255) / 256), (unsigned)P.nphase);
-    seg_desc_kernel<<<g, 256, 0, s>>>(off, nseg, segK, segR, counts, totals, L.per_phase, desc);
-    st = chk(cudaGetLastError(), "seg_desc");
-  }
+  mms_status st = chk(launch_k(seg_plan_kernel, dim3((unsigned)((nseg + 255) / 256)), dim3(256), 0, s,
+                               true, off, nseg, (unsigned long long)total_n, P, segK, segR, counts),
+                      "seg_plan");
+  if (st == MMS_OK)
+    st = chk(launch_k(seg_scan_kernel, dim3((unsigned)P.nphase), dim3(1024), 0, s, true, counts, nseg,
+                      totals, static_cast<const int*>(segK), dev_err, clear_status ? 1 : 0),
+             "seg_scan");
+  if (st == MMS_OK)
+    st = chk(launch_k(seg_desc_kernel, dim3((unsigned)((L.per_phase + 255) / 256), (unsigned)P.nphase),
+                      dim3(256), 0, s, true, off, nseg, static_cast<const int*>(segK),
+                      static_cast<const int*>(segR), static_cast<const int*>(counts),
+                      static_cast<const int*>(totals), L.per_phase, desc),
+             "seg_desc");
   void* bufA = pairs ? (void*)(ws + L.tmp0) : d_keys;     // where every segment ends
   void* bufB = pairs ? (void*)(ws + L.tmp1) : (void*)(ws + L.tmp0);
   if (st == MMS_OK && pairs)

@@ -18,7 +18,7 @@ __global__ void __launch_bounds__(WARPS * 32, (TileMinBlocks<KeyT, WARPS>::value
   griddep_wait();                                 // the keys: whatever ran before on the stream
   griddep_launch_dependents();                    // the first splitter may get resident early
   clear_status_word(status);
-  tile_sort_tile<KeyT, WARPS, XIN>(in, out, n, (long long)blockIdx.x * T, XOUT, smem_raw);
+  tile_sort_tile<KeyT, WARPS, XIN, sizeof(KeyT) == 4>(in, out, n, (long long)blockIdx.x * T, XOUT, smem_raw);
 }
 
 // Base case of the key-value sort: 32-bit keys -> sorted tiles of unique
@@ -32,7 +32,7 @@ __global__ void __launch_bounds__(WARPS * 32, (TileMinBlocks<uint64_t, WARPS>::v
   griddep_wait();
   griddep_launch_dependents();
   clear_status_word(status);
-  tile_sort_composite_tile<WARPS, XIN>(in, out, n, (long long)blockIdx.x * T, 0, smem_raw);
+  tile_sort_composite_tile<WARPS, XIN, false>(in, out, n, (long long)blockIdx.x * T, 0, smem_raw);
 }
 
 size_t tile_sort_smem_bytes(int key_bytes, int warps) {
