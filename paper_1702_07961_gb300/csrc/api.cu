@@ -432,9 +432,11 @@ mms_status mms_sort_keys(mms_key_type kt, void* d_keys, size_t n, void* d_ws, si
 // The 4-byte key-value sort on the composite buffers of layout L (the values
 // are copied first, so d_keys / d_values are overwritten only by the last
 // kernel): composite base case, merge rounds, key write-back and value gather.
+// d_values == NULL (a pass of the 8-byte sort): no values, and the sorted composites
+// are left in the buffer *sorted names instead.
 static mms_status pairs32_run(bool is_f32, void* d_keys, uint32_t* d_values, size_t n,
                               unsigned char* ws, const WsLayout& L, bool clear, cudaStream_t s,
-                              const mms_options* opt, int& ev) {
+                              const mms_options* opt, int& ev, void** sorted = nullptr) {
   int* dev_err = reinterpret_cast<int*>(ws);
   void* comp[2] = {ws + L.comp0_off, ws + L.comp1_off};
   void* vcopy = ws + L.vals_off;
@@ -457,8 +459,11 @@ static mms_status pairs32_run(bool is_f32, void* d_keys, uint32_t* d_values, siz
   };
   mms_status st = MMS_OK;
   mark();
-  cudaError_t ce = cudaMemcpyAsync(vcopy, d_values, n * sizeof(uint32_t), cudaMemcpyDeviceToDevice, s);
-  if (ce != cudaSuccess) st = cuda_fail(ce, "copy of the values");
+  if (d_values) {
+    const cudaError_t ce =
+        cudaMemcpyAsync(vcopy, d_values, n * sizeof(uint32_t), cudaMemcpyDeviceToDevice, s);
+    if (ce != cudaSuccess) st = cuda_fail(ce, "copy of the values");
+  }
   if (st == MMS_OK)
     st = check_launch(mms::launch_tile_sort_composite(tw, is_f32, d_keys, comp[0], (long long)n,
                                                       clear ? dev_err : nullptr, s),
@@ -484,7 +489,8 @@ static mms_status pairs32_run(bool is_f32, void* d_keys, uint32_t* d_values, siz
     cur = 1 - cur;
     run_len *= K[r];
   }
-  if (st == MMS_OK)
+  if (sorted) *sorted = comp[cur];
+  if (st == MMS_OK && d_values)
     st = check_launch(mms::launch_pairs_finalize(is_f32, comp[cur], vcopy, d_keys, d_values,
                                                  (long long)n, s), "pairs_finalize");
   mark();
@@ -533,18 +539,17 @@ mms_status mms_sort_pairs_ex(mms_key_type kt, void* d_keys, uint32_t* d_values, 
     void* perm = ws + L.perm_off;
     void* kcopy = ws + L.kcopy_off;
     void* vcopy = ws + L.vcopy_off;
-    st = check_launch(mms::launch_u64_pairs_split(d_keys, d_values, half, perm, kcopy, vcopy,
+    void* comp = nullptr;
+    st = check_launch(mms::launch_u64_pairs_split(d_keys, d_values, half, nullptr, kcopy, vcopy,
                                                   (long long)n, s), "key-value split (8-byte keys)");
+    if (st == MMS_OK) st = pairs32_run(false, half, nullptr, n, ws, L, true, s, opt, ev, &comp);
     if (st == MMS_OK)
-      st = pairs32_run(false, half, static_cast<uint32_t*>(perm), n, ws, L, true, s, opt, ev);
-    if (st == MMS_OK)
-      st = check_launch(mms::launch_u64_pairs_hi(kcopy, perm, half, (long long)n, s),
+      st = check_launch(mms::launch_u64_pairs_mid(comp, kcopy, perm, half, (long long)n, s),
                         "key-value high halves (8-byte keys)");
+    if (st == MMS_OK) st = pairs32_run(false, half, nullptr, n, ws, L, false, s, opt, ev, &comp);
     if (st == MMS_OK)
-      st = pairs32_run(false, half, static_cast<uint32_t*>(perm), n, ws, L, false, s, opt, ev);
-    if (st == MMS_OK)
-      st = check_launch(mms::launch_u64_pairs_final(kcopy, vcopy, perm, d_keys, d_values,
-                                                    (long long)n, s),
+      st = check_launch(mms::launch_u64_pairs_out(comp, perm, kcopy, vcopy, d_keys, d_values,
+                                                  (long long)n, s),
                         "key-value permutation (8-byte keys)");
   }
   if (owned) st = release_workspace(d_ws, s, st);

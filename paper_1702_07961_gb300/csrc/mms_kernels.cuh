@@ -87,12 +87,18 @@ cudaError_t launch_pairs_finalize(bool xout, const void* comp64, const void* val
                                   void* keys_out, void* vals_out, long long n, cudaStream_t s);
 
 // Key-value sort of 8-byte keys as two stable 4-byte passes (low half, then
-// high half): pass inputs, the high halves in pass-1 order, and the final
-// permutation of keys and values.
+// high half): pass inputs (perm may be NULL), the high halves in pass-1 order,
+// and the final permutation of keys and values; mid and out are the latter two
+// straight from the passes' composites.
 cudaError_t launch_u64_pairs_split(const void* keys, const void* vals, void* lo, void* perm,
                                    void* kcopy, void* vcopy, long long n, cudaStream_t s);
 cudaError_t launch_u64_pairs_hi(const void* kcopy, const void* perm, void* hi, long long n,
                                 cudaStream_t s);
+cudaError_t launch_u64_pairs_mid(const void* comp, const void* kcopy, void* perm, void* hi,
+                                 long long n, cudaStream_t s);
+cudaError_t launch_u64_pairs_out(const void* comp, const void* perm, const void* kcopy,
+                                 const void* vcopy, void* keys, void* vals, long long n,
+                                 cudaStream_t s);
 cudaError_t launch_u64_pairs_final(const void* kcopy, const void* vcopy, const void* perm,
                                    void* keys, void* vals, long long n, cudaStream_t s);
 

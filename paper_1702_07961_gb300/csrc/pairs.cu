@@ -70,7 +70,11 @@ cudaError_t launch_pairs_finalize(bool xout, const void* comp64, const void* val
 // position list by the high 32 key bits of the items it names.  Equal high
 // halves keep pass 1's order, which is by (low half, position), so the final
 // list is ordered by (key, position): the stable key order.  These kernels
-// prepare the passes and apply the final permutation.
+// prepare the passes and apply the final permutation.  A batch runs each pass as a
+// whole key-value sort (split, hi, final).  One array leaves each pass's result
+// as composites, whose low words are all that is wanted: the kernel between the
+// passes and the one after them read those, where the passes would write keys
+// nobody reads and gather positions that two more kernels gather through.
 
 __global__ void __launch_bounds__(256)
     u64_split_kernel(const uint64_t* __restrict__ keys, const uint32_t* __restrict__ vals,
@@ -81,7 +85,7 @@ __global__ void __launch_bounds__(256)
   for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += stride) {
     const uint64_t k = keys[i];
     lo[i] = (uint32_t)k;
-    perm[i] = (uint32_t)(pos0 + i);
+    if (perm != nullptr) perm[i] = (uint32_t)(pos0 + i);
     kcopy[i] = k;
     vcopy[i] = vals[i];
   }
@@ -102,6 +106,33 @@ __global__ void __launch_bounds__(256)
   const long long stride = (long long)gridDim.x * blockDim.x;
   for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += stride) {
     const long long p = (long long)perm[i] - pos0;
+    keys[i] = kcopy[p];
+    vals[i] = vcopy[p];
+  }
+}
+
+// Between the passes of one array, whose first pass sorts positions: item i of
+// the low pass is at position p of the array; perm[i] = p and the high half of its key.
+__global__ void __launch_bounds__(256)
+    u64_mid_kernel(const uint64_t* __restrict__ comp, const uint64_t* __restrict__ kcopy,
+                   uint32_t* __restrict__ perm, uint32_t* __restrict__ hi, long long n) {
+  const long long stride = (long long)gridDim.x * blockDim.x;
+  for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += stride) {
+    const uint32_t p = (uint32_t)comp[i];
+    perm[i] = p;
+    hi[i] = (uint32_t)(kcopy[p] >> 32);
+  }
+}
+
+// After the second pass: item i is the one the first pass put at place q, which is
+// at position perm[q] of the array.
+__global__ void __launch_bounds__(256)
+    u64_out_kernel(const uint64_t* __restrict__ comp, const uint32_t* __restrict__ perm,
+                   const uint64_t* __restrict__ kcopy, const uint32_t* __restrict__ vcopy,
+                   uint64_t* __restrict__ keys, uint32_t* __restrict__ vals, long long n) {
+  const long long stride = (long long)gridDim.x * blockDim.x;
+  for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += stride) {
+    const uint32_t p = perm[(uint32_t)comp[i]];
     keys[i] = kcopy[p];
     vals[i] = vcopy[p];
   }
@@ -139,6 +170,26 @@ cudaError_t launch_u64_pairs_final(const void* kcopy, const void* vcopy, const v
       static_cast<const uint64_t*>(kcopy), static_cast<const uint32_t*>(vcopy),
       static_cast<const uint32_t*>(perm), static_cast<uint64_t*>(keys),
       static_cast<uint32_t*>(vals), n, 0);
+  return cudaGetLastError();
+}
+
+cudaError_t launch_u64_pairs_mid(const void* comp, const void* kcopy, void* perm, void* hi,
+                                 long long n, cudaStream_t s) {
+  if (n <= 0) return cudaSuccess;
+  u64_mid_kernel<<<grid_for(n), 256, 0, s>>>(
+      static_cast<const uint64_t*>(comp), static_cast<const uint64_t*>(kcopy),
+      static_cast<uint32_t*>(perm), static_cast<uint32_t*>(hi), n);
+  return cudaGetLastError();
+}
+
+cudaError_t launch_u64_pairs_out(const void* comp, const void* perm, const void* kcopy,
+                                 const void* vcopy, void* keys, void* vals, long long n,
+                                 cudaStream_t s) {
+  if (n <= 0) return cudaSuccess;
+  u64_out_kernel<<<grid_for(n), 256, 0, s>>>(
+      static_cast<const uint64_t*>(comp), static_cast<const uint32_t*>(perm),
+      static_cast<const uint64_t*>(kcopy), static_cast<const uint32_t*>(vcopy),
+      static_cast<uint64_t*>(keys), static_cast<uint32_t*>(vals), n);
   return cudaGetLastError();
 }
 
