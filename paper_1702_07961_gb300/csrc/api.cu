@@ -108,21 +108,23 @@ bool valid_base_items(int key_bytes, int tw, int base_items) {
 // Fanouts of the merge rounds.  Sec. 6.2 tunes K per platform by
 // measurement; here the planner picks, per sort, the sequence of power-of-two
 // fanouts that minimises a cost model measured on GB300.  A round of fanout K
-// over n items costs about c0 + n * c1[K], where c1 is the merge pass plus
+// over n items costs about c0[K] + n * c1[K], where c1 is the merge pass plus
 // splitter time per item at n = 10^8 over the rounds that merged K runs per
 // group (bench.py --workload sweep, fitted by autotune.fit_plan_costs) and c0
-// the fixed cost of its two launches.  A last round over fewer runs builds
+// what a splitter and a merge pass of a few tiles take (10^5 u32 keys: 4.5 +
+// 6.4, 6.4 + 8.6, 6.8 + 11.3, 8.7 + 16.8 and 12.7 + 16.9 us), which the larger fanouts earn
+// back as one round instead of two.  A last round over fewer runs builds
 // its tree over those runs only, so it costs what a round of the next power
 // of two does.  Merge levels cost about the same for
 // K = 4..16, so the optimum first minimises the tree levels ceil(log2 runs)
-// and then the rounds (e.g. (16,16,8,8) for 10^8 4-byte keys).  The choice is
+// and then the rounds (e.g. (16,16,16,4) for 10^8 4-byte keys).  The choice is
 // a coin-change dynamic program over log2 of the coverage.  opt->fanout fixes
 // every round's K instead; the result does not depend on the plan.
 namespace plan_model {
 // ms per 10^8 items of one round (merge pass + splitter), for K = 2, 4, 8, 16, 32
-constexpr double kCost4[5] = {0.221, 0.332, 0.465, 0.621, 1.001};   // 4-byte keys
-constexpr double kCost8[5] = {0.466, 0.727, 1.035, 1.566, 2.873};   // 8-byte keys / composites
-constexpr double kLaunchMs = 0.010;                                 // two launches per round
+constexpr double kCost4[5] = {0.194, 0.312, 0.444, 0.567, 0.805};   // 4-byte keys
+constexpr double kCost8[5] = {0.419, 0.653, 0.953, 1.403, 2.400};   // 8-byte keys / composites
+constexpr double kLaunchMs[5] = {0.011, 0.015, 0.018, 0.023, 0.028};   // a round of a few tiles
 }  // namespace plan_model
 
 int plan_rounds(int key_bytes, size_t n, const mms_options* opt, int* K, int maxr) {
@@ -154,7 +156,7 @@ int plan_rounds(int key_bytes, size_t n, const mms_options* opt, int* K, int max
     pick[l] = 1;
     for (int b = 1; b <= 5; ++b) {
       const int rest = l - b > 0 ? l - b : 0;
-      const double c = best[rest] + plan_model::kLaunchMs + scale * c1[b - 1];
+      const double c = best[rest] + plan_model::kLaunchMs[b - 1] + scale * c1[b - 1];
       if (c < best[l]) {
         best[l] = c;
         pick[l] = b;
