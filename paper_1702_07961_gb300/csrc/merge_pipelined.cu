@@ -9,7 +9,7 @@
 // the third buffer.  Barriers (mbarriers in shared memory):
 //   full[b]  -- two arrivals and the bulk copies' bytes: the producer's
 //              expect-tx arrival as it starts the copies, and its arrival once
-//              the node table and the plainly loaded items are written;
+//              the block list and the plainly loaded items are written;
 //   empty[b] -- one arrival: the merging warps release p(q) when tile q is
 //              stored, which is the buffer tile q + 2 is staged into.
 // The producer's k-th wait on empty[b] and the merging warps' wait on
@@ -109,7 +109,7 @@ __global__ void __launch_bounds__((WARPS + 1) * 32, 2)
       if (lane == 0) {
         // A rejected plan started no copies and made no expect-tx arrival.
         if (ctl[kCtlErr]) mbar_arrive_plain(&full[b]);
-        mbar_arrive_plain(&full[b]);              // publishes the node table and plain loads
+        mbar_arrive_plain(&full[b]);              // publishes the block list and plain loads
       }
       staged = q + 1;
     }

@@ -7,8 +7,8 @@
 // a warp makes is 32 consecutive items (any base: one bank each), a row of 32
 // items whose 16-byte chunks are XOR-swizzled by the row index, a 16-byte
 // chunk whose position is XOR-permuted by the lane id, or a probe at an odd
-// stride -- never a data-dependent gather -- so no input can cause a bank
-// conflict.
+// stride (two searches' probes at once: at most two to a bank) -- never a
+// data-dependent gather -- so no input can cause bank conflicts.
 #pragma once
 
 #include <cuda_runtime.h>

@@ -2,8 +2,8 @@
 // their tile geometry.  A tile is S = 1024 * tile_warps items; the base case
 // sorts tiles of S keys and every merge round writes output tiles of S keys.
 // Defaults: 8 warps (8192 keys) for 4-byte keys, 4 warps (4096 keys) for
-// 8-byte keys, so that three CTAs' shared memory (two tile buffers each) fit
-// in one SM.
+// 8-byte keys, so that three merge CTAs' shared memory (two level buffers each)
+// fit in one SM.
 #pragma once
 
 #include <cuda_runtime.h>
@@ -27,9 +27,9 @@ constexpr int kDevOk = 0;
 constexpr int kDevErrTimeout = 1;       // an mbarrier wait ran out of its bound
 constexpr int kDevErrInternal = 2;      // a consistency check failed
 
-// CTAs per SM the tile kernels are compiled for (register budget): three
-// CTAs of 8 warps (4-byte keys) or of 4 warps (8-byte keys), whose shared
-// memory (two tile buffers each, about 66 KB) fits three to an SM.
+// CTAs per SM the merge pass is compiled for (register budget): three CTAs of
+// 8 warps (4-byte keys) or of 4 warps (8-byte keys), whose shared memory (two
+// level buffers each, 67 to 76 KB) fits three to an SM.
 template <typename KeyT, int WARPS>
 struct MinBlocks {
   static constexpr int value = 3;
