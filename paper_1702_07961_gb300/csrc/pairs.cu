@@ -11,6 +11,15 @@
 
 namespace mms {
 
+// The position a composite names, kept below n (last = n - 1).  Every composite
+// of a sort that went well names one; after a device error (a batch whose offsets
+// leave items out, a merge tile that gave up) a place may hold whatever was in the
+// workspace, and the gathers must stay inside their arrays all the same.  One
+// minimum an item, next to a gather: 3 * 10^7 pairs take the same time with it.
+__device__ __forceinline__ uint32_t item_position(uint64_t c, uint32_t last) {
+  return min((uint32_t)c, last);
+}
+
 template <bool XOUT>
 __global__ void __launch_bounds__(256)
     pairs_finalize_kernel(const uint64_t* __restrict__ comp, const uint32_t* __restrict__ vals_src,
@@ -20,6 +29,7 @@ __global__ void __launch_bounds__(256)
   // may start at any 4-byte offset), one item at a time otherwise.
   const bool vec = (((uintptr_t)keys_out | (uintptr_t)vals_out) & 15u) == 0;
   const long long nq = vec ? n / 4 : 0;
+  const uint32_t last = (uint32_t)(n - 1);
   const long long stride = (long long)gridDim.x * blockDim.x;
   for (long long q = (long long)blockIdx.x * blockDim.x + threadIdx.x; q < nq; q += stride) {
     // Composites and results pass through once and are marked so: the L2 is left to the
@@ -32,7 +42,7 @@ __global__ void __launch_bounds__(256)
     for (int i = 0; i < 4; ++i) {
       k[i] = (uint32_t)(c[i] >> 32);
       if (XOUT) k[i] = ordered_to_f32(k[i]);
-      v[i] = __ldg(vals_src + (uint32_t)c[i]);
+      v[i] = __ldg(vals_src + item_position(c[i], last));
     }
     __stcs(reinterpret_cast<uint4*>(keys_out) + q, make_uint4(k[0], k[1], k[2], k[3]));
     __stcs(reinterpret_cast<uint4*>(vals_out) + q, make_uint4(v[0], v[1], v[2], v[3]));
@@ -42,7 +52,7 @@ __global__ void __launch_bounds__(256)
     uint32_t k = (uint32_t)(c >> 32);
     if (XOUT) k = ordered_to_f32(k);
     keys_out[i] = k;
-    vals_out[i] = vals_src[(uint32_t)c];
+    vals_out[i] = vals_src[item_position(c, last)];
   }
 }
 
@@ -118,9 +128,10 @@ __global__ void __launch_bounds__(256)
 __global__ void __launch_bounds__(256)
     u64_mid_kernel(const uint64_t* __restrict__ comp, const uint64_t* __restrict__ kcopy,
                    uint32_t* __restrict__ perm, uint32_t* __restrict__ hi, long long n) {
+  const uint32_t last = (uint32_t)(n - 1);
   const long long stride = (long long)gridDim.x * blockDim.x;
   for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += stride) {
-    const uint32_t p = (uint32_t)comp[i];
+    const uint32_t p = item_position(comp[i], last);
     perm[i] = p;
     hi[i] = (uint32_t)(kcopy[p] >> 32);
   }
@@ -132,9 +143,10 @@ __global__ void __launch_bounds__(256)
     u64_out_kernel(const uint64_t* __restrict__ comp, const uint32_t* __restrict__ perm,
                    const uint64_t* __restrict__ kcopy, const uint32_t* __restrict__ vcopy,
                    uint64_t* __restrict__ keys, uint32_t* __restrict__ vals, long long n) {
+  const uint32_t last = (uint32_t)(n - 1);
   const long long stride = (long long)gridDim.x * blockDim.x;
   for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += stride) {
-    const uint32_t p = perm[(uint32_t)__ldcs(comp + i)];
+    const uint32_t p = perm[item_position(__ldcs(comp + i), last)];
     __stcs(keys + i, kcopy[p]);
     __stcs(vals + i, vcopy[p]);
   }
