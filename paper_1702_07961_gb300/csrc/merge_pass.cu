@@ -34,9 +34,10 @@ template <typename KeyT, int WARPS, bool XOUT, bool PART = false>
 static cudaError_t launch_merge_t(long long S, const void* in, void* out, long long n,
                                   long long run_len, int K, const long long* table, int* dev_err,
                                   cudaStream_t s, bool test_timeout, bool pdl) {
-  const size_t smem = PART ? MergeGeom<KeyT, WARPS>::bytes_partition(K) : MergeGeom<KeyT, WARPS>::bytes(K);
+  using G = MergeGeom<KeyT, WARPS>;
+  const size_t smem = PART ? G::bytes_partition(K) : G::bytes(K);
   auto k = merge_pass_kernel<KeyT, WARPS, XOUT, PART>;
-  cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  cudaError_t e = set_smem_limit(k, PART ? G::bytes_partition(kMaxFanout) : G::bytes(kMaxFanout));
   if (e != cudaSuccess) return e;
   if (S < kBlockItems || S > (long long)WARPS * kBlockItems || S % kBlockItems) return cudaErrorInvalidValue;
   const long long ntiles = num_tiles(S, n, run_len, K);

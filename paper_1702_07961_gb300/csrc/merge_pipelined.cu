@@ -157,7 +157,7 @@ cudaError_t launch_t(const void* in, void* out, long long n, long long run_len, 
                      const long long* table, int* dev_err, cudaStream_t s, bool pdl) {
   const size_t smem = PipeGeom<KeyT, WARPS>::bytes(K);
   auto k = merge_pipelined_kernel<KeyT, WARPS, XOUT>;
-  cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  cudaError_t e = set_smem_limit(k, PipeGeom<KeyT, WARPS>::bytes(kMaxFanout));
   if (e != cudaSuccess) return e;
   const long long S = 1024ll * WARPS;
   const long long ntiles = num_tiles(S, n, run_len, K);

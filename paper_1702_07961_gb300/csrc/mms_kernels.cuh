@@ -150,6 +150,16 @@ cudaError_t launch_k(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t sme
   return e;
 }
 
+// A kernel's dynamic shared-memory limit belongs to the process, so it is always set
+// to the same value, what the kernel takes for the largest fanout: a limit of one
+// call's own size would make a launch from another thread between this and the
+// call's launch fail.  What a launch asks for, and with it the CTAs that fit an
+// SM, stays the call's own.
+template <typename Kern>
+cudaError_t set_smem_limit(Kern kernel, size_t max_bytes) {
+  return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)max_bytes);
+}
+
 // Output tiles of a round: every group of K runs (K * run_len items, the last
 // group possibly short) is cut into tiles of S items, the last tile of every
 // group possibly short.

@@ -436,7 +436,7 @@ int sm_count() {
   return sms;
 }
 
-// Raises a kernel's dynamic shared-memory limit, except while `s` is being
+// Sets a kernel's dynamic shared-memory limit, except while `s` is being
 // captured into a graph: the capture is preceded by a preparing pass that
 // sets every attribute (attribute calls are not stream work).
 template <typename Kern>
@@ -445,7 +445,7 @@ cudaError_t set_smem(Kern k, size_t bytes, cudaStream_t s) {
   cudaError_t e = cudaStreamIsCapturing(s, &cs);
   if (e != cudaSuccess) return e;
   if (cs != cudaStreamCaptureStatusNone) return cudaSuccess;
-  return cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+  return set_smem_limit(k, bytes);
 }
 
 template <typename Kern>
@@ -518,13 +518,18 @@ size_t seg_merge_bar_off(int kmax) {
 }
 
 template <typename KeyT, int WARPS>
+size_t seg_merge_max_smem() {
+  return seg_merge_bar_off<KeyT, WARPS>(kMaxFanout) + 16 + kMergeCtlBytes;
+}
+
+template <typename KeyT, int WARPS>
 cudaError_t launch_seg_merge(void* a, void* b, const Desc* desc, const int* total,
                              long long upper, int r, bool is_f32, int kmax,
                              const long long* table, int* dev_err, cudaStream_t s) {
   auto k = seg_merge_kernel<KeyT, WARPS>;
   const size_t bar_off = seg_merge_bar_off<KeyT, WARPS>(kmax);
   const size_t smem = bar_off + 16 + kMergeCtlBytes;
-  cudaError_t e = set_smem(k, smem, s);
+  cudaError_t e = set_smem(k, seg_merge_max_smem<KeyT, WARPS>(), s);
   unsigned grid = 1;
   if (e == cudaSuccess) e = persistent_grid(k, WARPS * 32, smem, upper, &grid);
   if (e != cudaSuccess) return e;
@@ -573,36 +578,31 @@ cudaError_t seg_round(int unit_bytes, int tw, bool is_f32, int kmax, bool small,
   return cudaErrorInvalidValue;
 }
 
-template <typename Kern>
-cudaError_t attr(Kern k, size_t bytes) {
-  return cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
-}
-
 // Sets the shared-memory attribute of every kernel a batch of this shape
 // launches (before a graph capture, during which attributes are not set).
-mms_status seg_prepare(mms_key_type kt, bool pairs, int tw, int kmax) {
+mms_status seg_prepare(mms_key_type kt, bool pairs, int tw) {
   cudaError_t e = cudaSuccess;
   const bool f = kt == MMS_KEY_F32;
   if (pairs) {
     const size_t t = tile_sort_smem_bytes(8, tw);
-    if (tw == 4) e = f ? attr(seg_tile_sort_composite_kernel<4, true>, t) : attr(seg_tile_sort_composite_kernel<4, false>, t);
-    if (tw == 2) e = f ? attr(seg_tile_sort_composite_kernel<2, true>, t) : attr(seg_tile_sort_composite_kernel<2, false>, t);
+    if (tw == 4) e = f ? set_smem_limit(seg_tile_sort_composite_kernel<4, true>, t) : set_smem_limit(seg_tile_sort_composite_kernel<4, false>, t);
+    if (tw == 2) e = f ? set_smem_limit(seg_tile_sort_composite_kernel<2, true>, t) : set_smem_limit(seg_tile_sort_composite_kernel<2, false>, t);
   } else if (kt == MMS_KEY_U64) {
     const size_t t = tile_sort_smem_bytes(8, tw);
-    if (tw == 4) e = attr(seg_tile_sort_kernel<uint64_t, 4, false>, t);
-    if (tw == 2) e = attr(seg_tile_sort_kernel<uint64_t, 2, false>, t);
+    if (tw == 4) e = set_smem_limit(seg_tile_sort_kernel<uint64_t, 4, false>, t);
+    if (tw == 2) e = set_smem_limit(seg_tile_sort_kernel<uint64_t, 2, false>, t);
   } else {
     const size_t t = tile_sort_smem_bytes(4, tw);
-    if (tw == 8) e = f ? attr(seg_tile_sort_kernel<uint32_t, 8, true>, t) : attr(seg_tile_sort_kernel<uint32_t, 8, false>, t);
-    if (tw == 4) e = f ? attr(seg_tile_sort_kernel<uint32_t, 4, true>, t) : attr(seg_tile_sort_kernel<uint32_t, 4, false>, t);
+    if (tw == 8) e = f ? set_smem_limit(seg_tile_sort_kernel<uint32_t, 8, true>, t) : set_smem_limit(seg_tile_sort_kernel<uint32_t, 8, false>, t);
+    if (tw == 4) e = f ? set_smem_limit(seg_tile_sort_kernel<uint32_t, 4, true>, t) : set_smem_limit(seg_tile_sort_kernel<uint32_t, 4, false>, t);
   }
   if (e == cudaSuccess) {
     if (pairs || kt == MMS_KEY_U64) {
-      if (tw == 4) e = attr(seg_merge_kernel<uint64_t, 4>, seg_merge_bar_off<uint64_t, 4>(kmax) + 16 + kMergeCtlBytes);
-      if (tw == 2) e = attr(seg_merge_kernel<uint64_t, 2>, seg_merge_bar_off<uint64_t, 2>(kmax) + 16 + kMergeCtlBytes);
+      if (tw == 4) e = set_smem_limit(seg_merge_kernel<uint64_t, 4>, seg_merge_max_smem<uint64_t, 4>());
+      if (tw == 2) e = set_smem_limit(seg_merge_kernel<uint64_t, 2>, seg_merge_max_smem<uint64_t, 2>());
     } else {
-      if (tw == 8) e = attr(seg_merge_kernel<uint32_t, 8>, seg_merge_bar_off<uint32_t, 8>(kmax) + 16 + kMergeCtlBytes);
-      if (tw == 4) e = attr(seg_merge_kernel<uint32_t, 4>, seg_merge_bar_off<uint32_t, 4>(kmax) + 16 + kMergeCtlBytes);
+      if (tw == 8) e = set_smem_limit(seg_merge_kernel<uint32_t, 8>, seg_merge_max_smem<uint32_t, 8>());
+      if (tw == 4) e = set_smem_limit(seg_merge_kernel<uint32_t, 4>, seg_merge_max_smem<uint32_t, 4>());
     }
   }
   return e == cudaSuccess ? MMS_OK : seg_fail(MMS_ERR_CUDA, cudaGetErrorString(e));
@@ -724,7 +724,7 @@ static mms_status seg_sort_impl(mms_key_type kt, void* d_keys, uint32_t* d_value
   for (int c = 0; c <= size_class(mx); ++c) kmax = P.class_fanout[c] > kmax ? P.class_fanout[c] : kmax;
   P.kmax = kmax;
 
-  if (prepare_only) return seg_prepare(kt, pairs, tw, kmax);
+  if (prepare_only) return seg_prepare(kt, pairs, tw);
 
   int ev = 0;
   auto mark = [&]() {

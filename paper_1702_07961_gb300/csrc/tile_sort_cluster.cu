@@ -210,7 +210,7 @@ template <int CL, bool XIN, bool XOUT>
 static cudaError_t launch_cluster_t(const void* in, void* out, long long n, cudaStream_t s) {
   const size_t smem = 2 * sizeof(uint32_t) * (size_t)(kCT + kTileSlack);   // two chunk buffers
   auto k = tile_sort_cluster_kernel<CL, XIN, XOUT>;
-  cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  cudaError_t e = set_smem_limit(k, smem);
   if (e != cudaSuccess) return e;
   const long long R = (long long)CL * kCT;
   const long long clusters = (n + R - 1) / R;
