@@ -60,8 +60,8 @@ struct PipeGeom {
 
 template <typename KeyT, int WARPS, bool XOUT>
 __global__ void __launch_bounds__((WARPS + 1) * 32, 2)
-    merge_pipelined_kernel(const KeyT* __restrict__ in, KeyT* __restrict__ out, long long n,
-                           long long run_len, int K, const long long* __restrict__ table,
+    merge_pipelined_kernel(const KeyT* in, KeyT* out, long long n,
+                           long long run_len, int K, const long long* table,
                            long long tpg, long long ntiles, int S, int* dev_err) {
   using P = PipeGeom<KeyT, WARPS>;
   constexpr int NT = WARPS * 32;                  // merging threads

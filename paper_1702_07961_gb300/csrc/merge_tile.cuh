@@ -98,8 +98,8 @@ inline size_t merge_pass_smem_bytes_impl(int key_bytes, int warps, int K, bool p
 // loads first thing, so they are in flight across the CTA's setup.
 __device__ __forceinline__ void merge_tile_pivots(long long n, long long run_len, int K,
                                                   long long g, long long j,
-                                                  const long long* __restrict__ lo_row,
-                                                  const long long* __restrict__ hi_row, int S,
+                                                  const long long* lo_row,
+                                                  const long long* hi_row, int S,
                                                   int lane, long long& lo, long long& hi) {
   const long long gstart = g * run_len * K;
   const long long grest = n - gstart;
@@ -128,7 +128,7 @@ __device__ __forceinline__ void merge_tile_pivots(long long n, long long run_len
 // two halves need only the segment lengths and spans, which both compute, so a
 // CTA can start the copies and build the table at the same time.
 template <typename KeyT, int WARPS>
-__device__ __forceinline__ void merge_plan_warp(const KeyT* __restrict__ in, long long n,
+__device__ __forceinline__ void merge_plan_warp(const KeyT* in, long long n,
                                                 long long run_len, int K, long long g,
                                                 long long j, long long lo, long long hi, int S,
                                                 KeyT* stage, int* ctl, uint64_t* bar, int lane,
@@ -328,7 +328,7 @@ __device__ __forceinline__ void merge_plan_warp(const KeyT* __restrict__ in, lon
 // place at once; their tile goes out by the bulk store.
 template <typename KeyT, int WARPS, typename Sync>
 __device__ __forceinline__ void merge_levels(KeyT* bufX, KeyT* bufY, const int* ctl,
-                                             KeyT* __restrict__ dstg, bool xout, Sync sync) {
+                                             KeyT* dstg, bool xout, Sync sync) {
   constexpr int E = Vec16<KeyT>::E;
   constexpr uint32_t RB = 32 * sizeof(KeyT);
   constexpr bool LINEAR = sizeof(KeyT) == 4;
@@ -470,7 +470,7 @@ __device__ __forceinline__ void merge_levels(KeyT* bufX, KeyT* bufY, const int* 
 // so every shared-memory access stays inside the warp's spans.
 template <typename KeyT, int WARPS, typename Sync>
 __device__ __forceinline__ void merge_partition_blocks(const KeyT* bufX, KeyT* bufY, const int* ctl,
-                                                       int* rows, KeyT* __restrict__ dstg, bool xout,
+                                                       int* rows, KeyT* dstg, bool xout,
                                                        int* dev_err, Sync sync) {
   constexpr int E = Vec16<KeyT>::E;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -587,10 +587,10 @@ __device__ __forceinline__ void merge_partition_blocks(const KeyT* bufX, KeyT* b
 // PARTITION: merge with the heap-free variant above instead of the CTA tree
 // (shared memory of MergeGeom::bytes_partition).
 template <typename KeyT, int WARPS, bool PARTITION = false>
-__device__ __forceinline__ bool merge_tile(const KeyT* __restrict__ in, KeyT* __restrict__ out,
+__device__ __forceinline__ bool merge_tile(const KeyT* in, KeyT* out,
                                            long long n, long long run_len, int K, long long g,
-                                           long long j, const long long* __restrict__ lo_row,
-                                           const long long* __restrict__ hi_row, bool xout,
+                                           long long j, const long long* lo_row,
+                                           const long long* hi_row, bool xout,
                                            int* dev_err, unsigned char* smem_raw, uint64_t* bar,
                                            unsigned phase, int S, bool test_timeout = false) {
   using G = MergeGeom<KeyT, WARPS>;

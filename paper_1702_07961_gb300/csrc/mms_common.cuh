@@ -925,14 +925,17 @@ __device__ __forceinline__ void set_device_error(int* err, int code) {
 }
 
 // ---------------------------------------------------------------------------
-// Programmatic dependent launch (sm_90 and later).  The sort's kernels after
-// the base case are launched with programmatic stream serialization: a grid
-// may be scheduled once every CTA of the kernel before it has started, so its
+// Programmatic dependent launch (sm_90 and later).  Most of the sort's kernels,
+// the first one among them, are launched with programmatic stream
+// serialization: a grid may be scheduled once every CTA of the kernel before it has started, so its
 // CTAs become resident while that kernel's last wave drains.
 // griddep_wait() then blocks until the previous grid has completed and its
 // memory is visible; every such kernel calls it before its first global
 // memory access (reads and writes alike).  For a normal launch both are
-// no-ops.
+// no-ops.  The kernel before may still be writing what such a kernel reads while the
+// latter already runs, so its pointers carry no __restrict__ and its loads are plain ones:
+// both that qualifier and the read-only path promise memory that does not change
+// while the kernel lives, and a load under that promise may be moved above the wait.
 // ---------------------------------------------------------------------------
 __device__ __forceinline__ void griddep_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void griddep_launch_dependents() {

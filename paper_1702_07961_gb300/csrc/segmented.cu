@@ -72,7 +72,7 @@ struct Desc {
 static_assert(sizeof(Desc) == 16, "descriptor is 16 bytes");
 
 __device__ __forceinline__ Desc load_desc(const Desc* d) {
-  const uint4 v = __ldg(reinterpret_cast<const uint4*>(d));
+  const uint4 v = *reinterpret_cast<const uint4*>(d);
   Desc r;
   r.base = (unsigned long long)v.x | ((unsigned long long)v.y << 32);
   r.n = v.z;
@@ -90,9 +90,9 @@ __device__ __forceinline__ Desc load_desc(const Desc* d) {
 constexpr int kBadSegment = 1 << 8;               // in segK: offsets or size out of bounds
 
 // One thread per segment: K, R and the tile count of every phase.
-__global__ void seg_plan_kernel(const unsigned long long* __restrict__ off, long long nseg,
-                                unsigned long long total_n, SegPlan P, int* __restrict__ segK,
-                                int* __restrict__ segR, int* __restrict__ counts) {
+__global__ void seg_plan_kernel(const unsigned long long* off, long long nseg,
+                                unsigned long long total_n, SegPlan P, int* segK,
+                                int* segR, int* counts) {
   griddep_wait();
   griddep_launch_dependents();
   const long long s = (long long)blockIdx.x * blockDim.x + threadIdx.x;
@@ -127,9 +127,9 @@ __global__ void seg_plan_kernel(const unsigned long long* __restrict__ off, long
 // One CTA per phase: exclusive scan of the phase's counts in place, total
 // into totals[phase].  Phase 0's CTA also sets the status word: to an error when a
 // segment is marked bad, else to 0 (`clear`) or not at all.
-__global__ void __launch_bounds__(1024) seg_scan_kernel(int* __restrict__ counts, long long nseg,
-                                                        int* __restrict__ totals,
-                                                        const int* __restrict__ segK, int* dev_err,
+__global__ void __launch_bounds__(1024) seg_scan_kernel(int* counts, long long nseg,
+                                                        int* totals,
+                                                        const int* segK, int* dev_err,
                                                         int clear) {
   __shared__ int warp_sums[32];
   __shared__ int carry_s;
@@ -181,10 +181,10 @@ __global__ void __launch_bounds__(1024) seg_scan_kernel(int* __restrict__ counts
 
 // One thread per potential tile of a phase: finds its segment (last one whose
 // offset is <= t) and writes the descriptor.
-__global__ void seg_desc_kernel(const unsigned long long* __restrict__ off, long long nseg,
-                                const int* __restrict__ segK, const int* __restrict__ segR,
-                                const int* __restrict__ offs, const int* __restrict__ totals,
-                                long long per_phase, Desc* __restrict__ desc) {
+__global__ void seg_desc_kernel(const unsigned long long* off, long long nseg,
+                                const int* segK, const int* segR,
+                                const int* offs, const int* totals,
+                                long long per_phase, Desc* desc) {
   griddep_wait();
   griddep_launch_dependents();
   const int p = blockIdx.y;
@@ -221,8 +221,8 @@ __global__ void seg_desc_kernel(const unsigned long long* __restrict__ off, long
 
 template <typename KeyT, int WARPS, bool XIN>
 __global__ void __launch_bounds__(WARPS * 32, (TileMinBlocks<KeyT, WARPS>::value))
-    seg_tile_sort_kernel(const KeyT* __restrict__ keys_in, KeyT* bufA, KeyT* bufB,
-                         const Desc* __restrict__ desc, const int* __restrict__ total,
+    seg_tile_sort_kernel(const KeyT* keys_in, KeyT* bufA, KeyT* bufB,
+                         const Desc* desc, const int* total,
                          long long per_phase) {
   extern __shared__ __align__(1024) unsigned char smem_raw[];
   constexpr int T = WARPS * kBlockItems;
@@ -240,9 +240,9 @@ __global__ void __launch_bounds__(WARPS * 32, (TileMinBlocks<KeyT, WARPS>::value
 
 template <int WARPS, bool XIN>
 __global__ void __launch_bounds__(WARPS * 32, (TileMinBlocks<uint64_t, WARPS>::value))
-    seg_tile_sort_composite_kernel(const uint32_t* __restrict__ keys_in, uint64_t* bufA,
-                                   uint64_t* bufB, const Desc* __restrict__ desc,
-                                   const int* __restrict__ total, long long per_phase) {
+    seg_tile_sort_composite_kernel(const uint32_t* keys_in, uint64_t* bufA,
+                                   uint64_t* bufB, const Desc* desc,
+                                   const int* total, long long per_phase) {
   extern __shared__ __align__(1024) unsigned char smem_raw[];
   constexpr int T = WARPS * kBlockItems;
   griddep_wait();
@@ -262,9 +262,9 @@ __global__ void __launch_bounds__(WARPS * 32, (TileMinBlocks<uint64_t, WARPS>::v
 // when the whole batch is below 2^31 items.
 template <typename KeyT, int K2MAX, typename Idx>
 __global__ void __launch_bounds__(128)
-    seg_splitter_kernel(const KeyT* bufA, const KeyT* bufB, const Desc* __restrict__ desc,
-                        const int* __restrict__ total, long long per_phase, long long S, int r,
-                        long long* __restrict__ table) {
+    seg_splitter_kernel(const KeyT* bufA, const KeyT* bufB, const Desc* desc,
+                        const int* total, long long per_phase, long long S, int r,
+                        long long* table) {
   const int cnt = (int)min((long long)*total, per_phase);
   const long long warps = (long long)gridDim.x * (blockDim.x >> 5);
   for (long long t = (long long)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); t < cnt;
@@ -295,9 +295,9 @@ __global__ void __launch_bounds__(128)
 
 template <typename KeyT, int WARPS>
 __global__ void __launch_bounds__(WARPS * 32, (MinBlocks<KeyT, WARPS>::value))
-    seg_merge_kernel(KeyT* bufA, KeyT* bufB, const Desc* __restrict__ desc,
-                     const int* __restrict__ total, long long per_phase, int r, bool is_f32,
-                     const long long* __restrict__ table, size_t bar_off, int* dev_err) {
+    seg_merge_kernel(KeyT* bufA, KeyT* bufB, const Desc* desc,
+                     const int* total, long long per_phase, int r, bool is_f32,
+                     const long long* table, size_t bar_off, int* dev_err) {
   extern __shared__ __align__(1024) unsigned char smem_raw[];
   constexpr int S = WARPS * kBlockItems;
   uint64_t* bar = reinterpret_cast<uint64_t*>(smem_raw + bar_off);

@@ -18,8 +18,8 @@ constexpr long long kSplitterPdlTiles = 192;
 
 template <typename KeyT, int K2, typename Idx>
 __global__ void __launch_bounds__(32 * kSplitterWarps)
-    splitter_kernel(const KeyT* __restrict__ in, long long n, long long run_len, int K,
-                    long long S, unsigned tpg, unsigned ntiles, long long* __restrict__ table) {
+    splitter_kernel(const KeyT* in, long long n, long long run_len, int K,
+                    long long S, unsigned tpg, unsigned ntiles, long long* table) {
   griddep_wait();                                 // the runs are the previous kernel's output
   griddep_launch_dependents();
   const unsigned t = blockIdx.x * kSplitterWarps + (threadIdx.x >> 5);

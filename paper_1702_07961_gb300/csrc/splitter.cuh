@@ -403,9 +403,9 @@ __device__ __forceinline__ Idx window_pivot(const KeyT* run, Idx rlen, Idx maxle
 // are uniform over the warp.  Idx is the type of the counts and positions of
 // the search: int when n < 2^31, long long otherwise.  K2: K rounded up to a power of two.
 template <typename KeyT, int K2, typename Idx = long long>
-__device__ __forceinline__ void splitter_row(const KeyT* __restrict__ in, long long n,
+__device__ __forceinline__ void splitter_row(const KeyT* in, long long n,
                                              long long run_len, int K, long long S, long long g,
-                                             long long j, long long* __restrict__ row) {
+                                             long long j, long long* row) {
   constexpr int SUB = 32 / K2;
   const int lane = threadIdx.x & 31;
   const int rr = lane / SUB;                    // run of this lane

@@ -12,7 +12,7 @@ __device__ __forceinline__ void clear_status_word(int* status) {
 
 template <typename KeyT, int WARPS, bool XIN, bool XOUT>
 __global__ void __launch_bounds__(WARPS * 32, (TileMinBlocks<KeyT, WARPS>::value))
-    tile_sort_kernel(const KeyT* __restrict__ in, KeyT* out, long long n, int* status) {
+    tile_sort_kernel(const KeyT* in, KeyT* out, long long n, int* status) {
   extern __shared__ __align__(1024) unsigned char smem_raw[];
   constexpr int T = WARPS * kBlockItems;
   griddep_wait();                                 // the keys: whatever ran before on the stream
@@ -25,7 +25,7 @@ __global__ void __launch_bounds__(WARPS * 32, (TileMinBlocks<KeyT, WARPS>::value
 // 64-bit composites (ordered key << 32 | position in the array).
 template <int WARPS, bool XIN>
 __global__ void __launch_bounds__(WARPS * 32, (TileMinBlocks<uint64_t, WARPS>::value))
-    tile_sort_composite_kernel(const uint32_t* __restrict__ in, uint64_t* out, long long n,
+    tile_sort_composite_kernel(const uint32_t* in, uint64_t* out, long long n,
                                int* status) {
   extern __shared__ __align__(1024) unsigned char smem_raw[];
   constexpr int T = WARPS * kBlockItems;

@@ -264,7 +264,7 @@ __device__ __forceinline__ bool tile_idle_warp(int m) {
 // `base` (32 per lane, any assignment; pads past n), through the float order
 // transform when XIN.
 template <typename KeyT, int WARPS, bool XIN>
-__device__ __forceinline__ void tile_load(const KeyT* __restrict__ in, long long n, long long base,
+__device__ __forceinline__ void tile_load(const KeyT* in, long long n, long long base,
                                           KeyT (&v)[32]) {
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const long long wbase = base + (long long)warp * kBlockItems;
@@ -277,7 +277,7 @@ __device__ __forceinline__ void tile_load(const KeyT* __restrict__ in, long long
     const typename V::T* src = reinterpret_cast<const typename V::T*>(in + wbase);
 #pragma unroll
     for (int q = 0; q < NV; ++q) {
-      const typename V::T x = __ldg(src + q * 32 + lane);
+      const typename V::T x = src[q * 32 + lane];
       KeyT t[V::E];
       V::unpack(x, t);
 #pragma unroll
@@ -298,7 +298,7 @@ __device__ __forceinline__ void tile_load(const KeyT* __restrict__ in, long long
 // Sorts the tile of 1024 * WARPS keys of in[0, n) that starts at `base` into
 // the same positions of out (in == out allowed): the CTA body of the base case.
 template <typename KeyT, int WARPS, bool XIN, bool SHORT>
-__device__ __forceinline__ void tile_sort_tile(const KeyT* __restrict__ in, KeyT* out, long long n,
+__device__ __forceinline__ void tile_sort_tile(const KeyT* in, KeyT* out, long long n,
                                                long long base, bool xout,
                                                unsigned char* smem_raw) {
   constexpr int T = WARPS * kBlockItems;
@@ -317,7 +317,7 @@ __device__ __forceinline__ void tile_sort_tile(const KeyT* __restrict__ in, KeyT
 // (ordered key << 32 | pos0 + position in the array), whose ascending order is the
 // stable key order; tiles of composites are then sorted like 64-bit keys.
 template <int WARPS, bool XIN, bool SHORT>
-__device__ __forceinline__ void tile_sort_composite_tile(const uint32_t* __restrict__ in,
+__device__ __forceinline__ void tile_sort_composite_tile(const uint32_t* in,
                                                          uint64_t* out, long long n,
                                                          long long base, long long pos0,
                                                          unsigned char* smem_raw) {
@@ -334,7 +334,7 @@ __device__ __forceinline__ void tile_sort_composite_tile(const uint32_t* __restr
       const uint4* src = reinterpret_cast<const uint4*>(in + wbase);
   #pragma unroll
       for (int q = 0; q < 8; ++q) {
-        const uint4 x = __ldg(src + q * 32 + lane);
+        const uint4 x = src[q * 32 + lane];
         const uint32_t k[4] = {x.x, x.y, x.z, x.w};
   #pragma unroll
         for (int c = 0; c < 4; ++c) {

@@ -184,7 +184,7 @@ __device__ __forceinline__ void cluster_level(int lv, uint32_t* cur, uint32_t* f
 // tile before the first cluster barrier, and clusters cover disjoint keys).
 template <int CL, bool XIN, bool XOUT>
 __global__ void __launch_bounds__(256, (MinBlocks<uint32_t, 8>::value))
-    tile_sort_cluster_kernel(const uint32_t* __restrict__ in, uint32_t* out, long long n) {
+    tile_sort_cluster_kernel(const uint32_t* in, uint32_t* out, long long n) {
   extern __shared__ __align__(1024) unsigned char smem_raw[];
   __shared__ int s_co[2];
   griddep_launch_dependents();                    // the first splitter may get resident early
