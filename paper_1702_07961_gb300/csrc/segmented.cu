@@ -260,8 +260,11 @@ __global__ void __launch_bounds__(WARPS * 32, (TileMinBlocks<uint64_t, WARPS>::v
 // K2MAX: the largest fanout of the batch's classes, rounded up to a power of
 // two (the code, and the registers, of larger ones are left out); Idx: int
 // when the whole batch is below 2^31 items.
+// Compiled for 32 warps an SM (64 registers), 4-byte keys with small fanouts for 40: 60
+// arrays of up to 2^20 keys are within 0.5% with 32, 40 or no bound, 2000 of them are
+// 4.37, 4.36 and 4.38 ms (u32), with K = 32 and nearly sorted keys 10.55, 10.69 and 10.81.
 template <typename KeyT, int K2MAX, typename Idx>
-__global__ void __launch_bounds__(128)
+__global__ void __launch_bounds__(128, (sizeof(KeyT) == 4 && K2MAX == 8 ? 10 : 8))
     seg_splitter_kernel(const KeyT* bufA, const KeyT* bufB, const Desc* desc,
                         const int* total, long long per_phase, long long S, int r,
                         long long* table) {

@@ -16,8 +16,14 @@ constexpr int kSplitterWarps = 4;
 // without, 66 with).
 constexpr long long kSplitterPdlTiles = 192;
 
+// CTAs per SM the splitter is compiled for: 40 warps (48 registers), 32 with more than 16
+// runs, whose window is twice as large.  The search waits for loads, so warps count: left
+// to itself the compiler takes 40 to 64 and spills some (6 * 10^6 pairs of 4-byte keys 411 -> 414
+// us, 10^8 u32 keys' splitters 262 -> 266); for 48 warps it spills more (268).
+constexpr int splitter_ctas(int k2) { return k2 == 32 ? 8 : 10; }
+
 template <typename KeyT, int K2, typename Idx>
-__global__ void __launch_bounds__(32 * kSplitterWarps)
+__global__ void __launch_bounds__(32 * kSplitterWarps, splitter_ctas(K2))
     splitter_kernel(const KeyT* in, long long n, long long run_len, int K,
                     long long S, unsigned tpg, unsigned ntiles, long long* table) {
   griddep_wait();                                 // the runs are the previous kernel's output

@@ -257,11 +257,19 @@ __device__ __forceinline__ Idx multiseq_pivot(const KeyT* run, Idx rlen, bool ac
 //     ones.  The 32 M windowed samples are sorted across the warp (bitonic
 //     merges of the windows, which are sorted already); the D-th largest is the
 //     threshold, and every lane compares its own samples with it.
-//   - A run whose whole window goes may have to give up more.  Of those runs
-//     the one whose lowest windowed sample is the largest loses its whole
-//     window for certain (samples not yet seen are all smaller), so it moves
-//     on by one window and the selection is repeated with D - W.  About 3% of
-//     the steps of 16 random runs do this, fewer with fewer runs.
+//   - A run whose whole window goes may have to give up more: it is deep.  Every run's
+//     coarser pivot left part of a sample behind, and where the runs overlap little (nearly
+//     sorted keys, few distinct ones) the one run that holds the boundary gives all of
+//     that back, up to D of its samples (D < 16 M).  Of the deep runs, that whose lowest windowed
+//     sample is the largest, r, loses its window for certain (samples not yet seen are all
+//     smaller).  Either it moves on by that window and the selection is repeated, or
+//     (kLongWindow) its next 16 M samples, more than it can lose, take the place of the
+//     lower half of the sorted order, which cannot reach the D largest, and one bitonic
+//     merge gives the threshold again; if another run is still deep then, all that lies above the
+//     largest of their lowest samples has been seen and goes for certain, and the step takes
+//     another turn.  About 1% of the steps of 16 random runs come here, 0.1% with 8, and most of
+//     those of nearly sorted ones, which took 3.2 loads a step with 16 runs moved a window a
+//     turn: 10^8 u32 keys with 1% of them swapped, splitters 631 -> 330 us.
 //   - The first stride is the least power of W / 2 at which every run has at most W
 //     samples; there top = len / s and the windows are all there is.
 //
@@ -269,11 +277,12 @@ __device__ __forceinline__ Idx multiseq_pivot(const KeyT* run, Idx rlen, bool ac
 //
 // What bounds it: up to about 3000 rows (one wave of warps) a chain of
 // log(run_len) / log(W / 2) steps, each a load (700 cycles and more) and a sort of
-// about as long; above that the 32 M sectors a step reads.  Stride halving took
-// log2(K * run_len) levels, each a load and about K / 2 arg-maxes of 250 cycles.  Both
-// splitters of 2^20 u32 keys 41 -> 25 us, the three of 16.8 * 10^6 85 -> 59 us, the
-// four of 10^8 304 -> 264 us.  Finding the threshold by quickselect instead of
-// sorting took 500 cycles a round of 5 to 7 rounds and was no faster than stride halving.
+// about as long; above that the 32 M sectors a step reads.  Against stride halving (log2(K *
+// run_len) levels, each a load and about K / 2 arg-maxes of 250 cycles) on random keys: both
+// splitters of 2^20 u32 keys 41 -> 25 us, the three of 16.8 * 10^6 85 -> 59 us, the four of
+// 3 * 10^8 926 -> 811 us, the five of 10^8 u64 567 -> 596 us.  Finding the threshold by
+// quickselect instead of sorting took 500 cycles a round of 5 to 7 rounds and was no faster
+// than stride halving.
 
 // Samples per lane.  More samples take fewer, longer steps and read more
 // sectors: with K = 8, 4 against 2 measured 12.3 against 18.4 us at 2^20 u32 keys and
@@ -315,6 +324,29 @@ __device__ __forceinline__ void window_sort(KeyT (&v)[M], int lane) {
   }
 }
 
+// Element `at` of the sorted windows.  In PTX, because a choice by a run-time index is
+// compiled as an array in local memory.
+template <int M>
+__device__ __forceinline__ uint32_t window_at(const uint32_t (&v)[M], int at) {
+  uint32_t t = v[0];
+#pragma unroll
+  for (int m = 1; m < M; ++m)
+    asm("{\n\t.reg .pred p;\n\tsetp.eq.s32 p, %2, %3;\n\tselp.b32 %0, %1, %0, p;\n\t}\n"
+        : "+r"(t)
+        : "r"(v[m]), "r"(at & (M - 1)), "r"(m));
+  return __shfl_sync(0xffffffffu, t, at / M);
+}
+template <int M>
+__device__ __forceinline__ uint64_t window_at(const uint64_t (&v)[M], int at) {
+  uint64_t t = v[0];
+#pragma unroll
+  for (int m = 1; m < M; ++m)
+    asm("{\n\t.reg .pred p;\n\tsetp.eq.s32 p, %2, %3;\n\tselp.b64 %0, %1, %0, p;\n\t}\n"
+        : "+l"(t)
+        : "l"(v[m]), "r"(at & (M - 1)), "r"(m));
+  return __shfl_sync(0xffffffffu, t, at / M);
+}
+
 // `run` and `rlen`: the run of this lane (lane / SUB) and its length, 0 past
 // the K runs; maxlen: an upper bound of the lengths; k <= their sum.  All 32
 // lanes call, k and maxlen uniform.  Returns the run's pivot on each of its
@@ -326,6 +358,10 @@ __device__ __forceinline__ Idx window_pivot(const KeyT* run, Idx rlen, Idx maxle
   constexpr int W = SUB * M;
   constexpr int B = W == 4 ? 1 : W == 8 ? 2 : W == 16 ? 3 : W == 32 ? 4 : 5;   // log2(W / 2)
   static_assert(W == (2 << B), "windows of 4 to 64 samples");
+  // Whether a deep run goes on by 16 M samples at once or by a window a turn.  With 8 runs it
+  // rarely moves twice; with 8-byte keys the code alone made small sorts slower (3 * 10^6 pairs
+  // of 8-byte keys 473 -> 491 us with K = 16, 6 * 10^6 900 -> 917 with K = 8).
+  constexpr bool kLongWindow = K2 >= 16 && sizeof(KeyT) == 4;
   const int lane = threadIdx.x & 31, sub = lane % SUB;
   if (k == 0) return 0;
   int sh = 0;
@@ -334,29 +370,23 @@ __device__ __forceinline__ Idx window_pivot(const KeyT* run, Idx rlen, Idx maxle
   for (;;) {
     int D = (int)(__reduce_add_sync(0xffffffffu, sub == 0 ? (unsigned)top : 0u) - (unsigned)(k >> sh));
     int gone = 0;
-    while (D > 0) {
+    // Sorted runs need K2 / 2 turns at most (D < K2 * W / 2, and another turn comes after W
+    // drops or more); after K2 the search gives up on runs that are not sorted.
+    for (int turn = 0; D > 0 && turn < K2; ++turn) {
       KeyT w[M], v[M];
-      int tot = 0;
 #pragma unroll
       for (int m = 0; m < M; ++m) {
         const Idx f = top - (Idx)(W - 1 - m - sub * M);
         w[m] = f >= 1 ? run[(f << sh) - 1] : KeyT(0);
         v[m] = w[m];
-        tot += __popc(__ballot_sync(0xffffffffu, f >= 1));
       }
-      unsigned X[M];
-      if (D >= tot) {                              // everything in the windows goes
-#pragma unroll
-        for (int m = 0; m < M; ++m) X[m] = __ballot_sync(0xffffffffu, top >= (Idx)(W - m - sub * M));
-      } else {
-        window_sort<W, M>(v, lane);
-        const int pos = 32 * M - D;                // the D largest start there
-        KeyT t = v[0];
-#pragma unroll
-        for (int m = 1; m < M; ++m) t = pos % M == m ? v[m] : t;
-        t = __shfl_sync(0xffffffffu, t, pos / M);
-        unsigned E[M];
-        int need = D, eq = 0;
+      window_sort<W, M>(v, lane);
+
+      // Drops the `need` largest of the windows and of `extra` equal samples of run r
+      // that lie below its window: sets gone, returns how many of the extra ones go.
+      auto drop = [&](KeyT t, int need, int extra, int r) {
+        unsigned X[M], E[M];
+        int eq = extra;
 #pragma unroll
         for (int m = 0; m < M; ++m) {
           X[m] = __ballot_sync(0xffffffffu, w[m] > t);
@@ -364,13 +394,19 @@ __device__ __forceinline__ Idx window_pivot(const KeyT* run, Idx rlen, Idx maxle
           need -= __popc(X[m]);
           eq += __popc(E[m]);
         }
-        if (need == eq) {
+        int left = extra;
+        if (need >= eq) {
 #pragma unroll
           for (int m = 0; m < M; ++m) X[m] |= E[m];
         } else {                                   // of equal keys, those of the later runs and places
-          int above = 0;
+          int above = lane / SUB < r ? extra : 0;
+          left = need;
 #pragma unroll
-          for (int m = 0; m < M; ++m) above += __popc(E[m] & ~(0xffffffffu >> (31 - lane)));
+          for (int m = 0; m < M; ++m) {
+            above += __popc(E[m] & ~(0xffffffffu >> (31 - lane)));
+            if (extra > 0) left -= __popc(E[m] >> (r * SUB));
+          }
+          left = left < 0 ? 0 : left < extra ? left : extra;
 #pragma unroll
           for (int m = M - 1; m >= 0; --m) {
             const bool mine = (E[m] >> lane) & 1u;
@@ -378,15 +414,58 @@ __device__ __forceinline__ Idx window_pivot(const KeyT* run, Idx rlen, Idx maxle
             above += mine;
           }
         }
-      }
-      gone = 0;
+        gone = 0;
 #pragma unroll
-      for (int m = 0; m < M; ++m) gone += __popc((X[m] >> (lane - sub)) & (unsigned)((1ull << SUB) - 1));
-      const bool deep = sub == 0 && gone == W && top > W;   // its lane holds the lowest sample
+        for (int m = 0; m < M; ++m) gone += __popc((X[m] >> (lane - sub)) & (unsigned)((1ull << SUB) - 1));
+        return left;
+      };
+
+      drop(window_at<M>(v, 32 * M - D), D, 0, -1);   // the D largest start there
+      bool deep = sub == 0 && gone == W && top > W;  // its lane holds the run's lowest sample
       if (!__any_sync(0xffffffffu, deep)) break;
-      const int r = (31 - __clz(lanes_with_max(0xffffffffu, deep, w[0]))) / SUB;
-      if (lane / SUB == r) top -= W;
-      D -= W;
+
+      const int at = 31 - __clz(lanes_with_max(0xffffffffu, deep, w[0]));
+      if constexpr (!kLongWindow) {
+        if (lane / SUB == at / SUB) top -= W;
+        D -= W;
+        gone = 0;
+        continue;
+      }
+      // Run r, that of the largest such sample, goes on below its window: the next 16 M
+      // samples (more than it can lose) take the place of the lower half.
+      const KeyT* rrun = reinterpret_cast<const KeyT*>(__shfl_sync(0xffffffffu, (unsigned long long)run, at));
+      const Idx below = __shfl_sync(0xffffffffu, top, at) - W;
+      KeyT x[M];
+#pragma unroll
+      for (int m = 0; m < M; ++m) {
+        const Idx f = below - (Idx)(16 * M - 1 - m - lane * M);
+        x[m] = lane < 16 && f >= 1 ? rrun[(f << sh) - 1] : KeyT(0);
+        v[m] = lane < 16 ? x[m] : v[m];
+      }
+      window_merge<32 * M, M>(v, lane);
+      const KeyT t = window_at<M>(v, 32 * M - D);
+      int more = 0, extra = 0;
+#pragma unroll
+      for (int m = 0; m < M; ++m) {
+        more += __popc(__ballot_sync(0xffffffffu, x[m] > t));
+        extra += __popc(__ballot_sync(0xffffffffu, x[m] == t && lane < 16 && below >= (Idx)(16 * M - m - lane * M)));
+      }
+      more += drop(t, D - more, extra, at / SUB);
+      deep = deep && gone == W && lane != at;
+      if (!__any_sync(0xffffffffu, deep)) {
+        if (lane / SUB == at / SUB) gone += more;
+        break;
+      }
+      // Another run may have to go on too.  All that lies above the largest of their
+      // lowest samples has been seen and goes for certain.
+      const int at2 = 31 - __clz(lanes_with_max(0xffffffffu, deep, w[0]));
+      const KeyT low = __shfl_sync(0xffffffffu, w[0], at2);
+      more = W;
+#pragma unroll
+      for (int m = 0; m < M; ++m) more += __popc(__ballot_sync(0xffffffffu, x[m] > low));
+      if (lane / SUB == at / SUB) top -= more;
+      if (lane / SUB == at2 / SUB) top -= W;
+      D -= more + W;
       gone = 0;
     }
     top -= gone;
