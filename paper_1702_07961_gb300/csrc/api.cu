@@ -224,10 +224,11 @@ mms_status alloc_workspace(void** d_ws, size_t bytes, cudaStream_t s) {
 
 // Ends a sort on a library-allocated workspace without waiting for it: the
 // status word goes to the per-device word, then the workspace is freed, both
-// in stream order.
-mms_status release_workspace(void* d_ws, cudaStream_t s, mms_status st) {
-  forward_status_kernel<<<1, 1, 0, s>>>(static_cast<const int*>(d_ws));
-  const cudaError_t e1 = cudaGetLastError();
+// in stream order.  `cleared`: what clears the word has been queued; a call that
+// failed before that leaves whatever the allocation held there, which is no error of a sort.
+mms_status release_workspace(void* d_ws, cudaStream_t s, mms_status st, bool cleared) {
+  if (cleared) forward_status_kernel<<<1, 1, 0, s>>>(static_cast<const int*>(d_ws));
+  const cudaError_t e1 = cleared ? cudaGetLastError() : cudaSuccess;
   const cudaError_t e2 = cudaFreeAsync(d_ws, s);
   if (st == MMS_OK && e1 != cudaSuccess) st = cuda_fail(e1, "status forwarding");
   if (st == MMS_OK && e2 != cudaSuccess) st = cuda_fail(e2, "workspace release");
@@ -370,9 +371,11 @@ mms_status mms_sort_keys_ex(mms_key_type kt, void* d_keys, size_t n, void* d_ws,
     if (as != MMS_OK) return as;
     owned = true;
   }
+  bool cleared = false;
   if (d_ws && cluster) {                                // else the base case clears it
     const mms_status cs = clear_status(d_ws, s);
-    if (cs != MMS_OK) return owned ? release_workspace(d_ws, s, cs) : cs;
+    if (cs != MMS_OK) return owned ? release_workspace(d_ws, s, cs, false) : cs;
+    cleared = true;
   }
   unsigned char* ws = static_cast<unsigned char*>(d_ws);
   int* dev_err = reinterpret_cast<int*>(ws);
@@ -401,6 +404,7 @@ mms_status mms_sort_keys_ex(mms_key_type kt, void* d_keys, size_t n, void* d_ws,
                                                         is_f32 && rounds == 0, d_keys, cur,
                                                         (long long)n, s),
                     "tile_sort");
+  if (st == MMS_OK) cleared = true;
   mark();
   for (int r = 0; r < rounds && st == MMS_OK; ++r) {
     const long long Sm = merge_tile_for(kb, tw, K[r], opt, n, run_len);
@@ -422,7 +426,7 @@ mms_status mms_sort_keys_ex(mms_key_type kt, void* d_keys, size_t n, void* d_ws,
     other = t;
     run_len *= K[r];
   }
-  if (owned) st = release_workspace(d_ws, s, st);
+  if (owned) st = release_workspace(d_ws, s, st, cleared);
   return st;
 }
 
@@ -435,9 +439,10 @@ mms_status mms_sort_keys(mms_key_type kt, void* d_keys, size_t n, void* d_ws, si
 // are copied first, so d_keys / d_values are overwritten only by the last
 // kernel): composite base case, merge rounds, key write-back and value gather.
 // d_values == NULL (a pass of the 8-byte sort): no values, and the sorted composites
-// are left in the buffer *sorted names instead.
+// are left in the buffer *sorted names instead.  cleared: whether the status word has been
+// cleared already; if not, the base case does.
 static mms_status pairs32_run(bool is_f32, void* d_keys, uint32_t* d_values, size_t n,
-                              unsigned char* ws, const WsLayout& L, bool clear, cudaStream_t s,
+                              unsigned char* ws, const WsLayout& L, bool& cleared, cudaStream_t s,
                               const mms_options* opt, int& ev, void** sorted = nullptr) {
   int* dev_err = reinterpret_cast<int*>(ws);
   void* comp[2] = {ws + L.comp0_off, ws + L.comp1_off};
@@ -468,8 +473,9 @@ static mms_status pairs32_run(bool is_f32, void* d_keys, uint32_t* d_values, siz
   }
   if (st == MMS_OK)
     st = check_launch(mms::launch_tile_sort_composite(tw, is_f32, d_keys, comp[0], (long long)n,
-                                                      clear ? dev_err : nullptr, s),
+                                                      cleared ? nullptr : dev_err, s),
                       "tile_sort (key-value)");
+  if (st == MMS_OK) cleared = true;
   mark();
   long long run_len = S;
   int cur = 0;
@@ -532,9 +538,10 @@ mms_status mms_sort_pairs_ex(mms_key_type kt, void* d_keys, uint32_t* d_values, 
   }
   unsigned char* ws = static_cast<unsigned char*>(d_ws);
   int ev = 0;
+  bool cleared = false;
   mms_status st = MMS_OK;
   if (kt != MMS_KEY_U64) {
-    st = pairs32_run(kt == MMS_KEY_F32, d_keys, d_values, n, ws, L, true, s, opt, ev);
+    st = pairs32_run(kt == MMS_KEY_F32, d_keys, d_values, n, ws, L, cleared, s, opt, ev);
   } else {
     // Two stable 4-byte passes, low half first (see pairs.cu).
     void* half = ws + L.half_off;
@@ -544,17 +551,17 @@ mms_status mms_sort_pairs_ex(mms_key_type kt, void* d_keys, uint32_t* d_values, 
     void* comp = nullptr;
     st = check_launch(mms::launch_u64_pairs_split(d_keys, d_values, half, nullptr, kcopy, vcopy,
                                                   (long long)n, s), "key-value split (8-byte keys)");
-    if (st == MMS_OK) st = pairs32_run(false, half, nullptr, n, ws, L, true, s, opt, ev, &comp);
+    if (st == MMS_OK) st = pairs32_run(false, half, nullptr, n, ws, L, cleared, s, opt, ev, &comp);
     if (st == MMS_OK)
       st = check_launch(mms::launch_u64_pairs_mid(comp, kcopy, perm, half, (long long)n, s),
                         "key-value high halves (8-byte keys)");
-    if (st == MMS_OK) st = pairs32_run(false, half, nullptr, n, ws, L, false, s, opt, ev, &comp);
+    if (st == MMS_OK) st = pairs32_run(false, half, nullptr, n, ws, L, cleared, s, opt, ev, &comp);
     if (st == MMS_OK)
       st = check_launch(mms::launch_u64_pairs_out(comp, perm, kcopy, vcopy, d_keys, d_values,
                                                   (long long)n, s),
                         "key-value permutation (8-byte keys)");
   }
-  if (owned) st = release_workspace(d_ws, s, st);
+  if (owned) st = release_workspace(d_ws, s, st, cleared);
   return st;
 }
 
