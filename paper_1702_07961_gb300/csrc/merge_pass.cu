@@ -5,10 +5,6 @@
 
 namespace mms {
 
-size_t merge_pass_smem_bytes(int key_bytes, int warps, int K) {
-  return merge_pass_smem_bytes_impl(key_bytes, warps, K);
-}
-
 template <typename KeyT, int WARPS, bool XOUT, bool PART>
 __global__ void __launch_bounds__(WARPS * 32, (PART ? kPartitionMinBlocks : MinBlocks<KeyT, WARPS>::value))
     merge_pass_kernel(const KeyT* in, KeyT* out, long long n,

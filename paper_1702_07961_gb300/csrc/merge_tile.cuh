@@ -58,7 +58,7 @@ constexpr size_t kMergeCtlBytes = sizeof(int) * kCtlInts;
 // alignment slack and 16 items of transpose slack per segment: a node that runs a
 // network has two segments at least, and its last block may use 31 items past
 // its end), and the odd tree levels' inputs; Y: the same spans, one buffer per
-// level parity.  Three CTAs fit an SM up to K = 32 (76464 of 76800 bytes with 8-byte keys).
+// level parity.  Three CTAs fit an SM up to K = 32.
 template <typename KeyT, int WARPS>
 struct MergeGeom {
   static constexpr int E = Vec16<KeyT>::E;
@@ -77,21 +77,9 @@ struct MergeGeom {
   static constexpr size_t kRowBytes = sizeof(int) * 32 * (WARPS + 3);
   __host__ __device__ static constexpr size_t bytes_partition(int K) { return bytes(K) + kRowBytes; }
 };
-
-inline size_t merge_pass_smem_bytes_impl(int key_bytes, int warps, int K, bool partition = false) {
-  if (key_bytes == 4) {
-    switch (warps) {
-      case 4: return partition ? MergeGeom<uint32_t, 4>::bytes_partition(K) : MergeGeom<uint32_t, 4>::bytes(K);
-      case 8: return partition ? MergeGeom<uint32_t, 8>::bytes_partition(K) : MergeGeom<uint32_t, 8>::bytes(K);
-    }
-  } else {
-    switch (warps) {
-      case 2: return partition ? MergeGeom<uint64_t, 2>::bytes_partition(K) : MergeGeom<uint64_t, 2>::bytes(K);
-      case 4: return partition ? MergeGeom<uint64_t, 4>::bytes_partition(K) : MergeGeom<uint64_t, 4>::bytes(K);
-    }
-  }
-  return 0;
-}
+// An SM's 228 KB, of which every CTA takes 1 KB beside its own.
+static_assert(3 * (MergeGeom<uint32_t, 8>::bytes(kMaxFanout) + 1024) <= 228 * 1024, "three CTAs an SM");
+static_assert(3 * (MergeGeom<uint64_t, 4>::bytes(kMaxFanout) + 1024) <= 228 * 1024, "three CTAs an SM");
 
 // Segment bounds of the tile in run `lane` (lanes < K): from the pivot rows,
 // or the run's ends for a group's first / last tile.  Warp 0 issues these

@@ -277,15 +277,46 @@ template <typename KeyT>
 __device__ __forceinline__ void lds_if_lt(KeyT& v, const KeyT* p, int idx, int lim) {
   lds_if_lt(v, smem_u32addr(p), idx, lim);
 }
-__device__ __forceinline__ uint32_t lds_key(const uint32_t* p) {
-  uint32_t v;
-  asm volatile("ld.shared.b32 %0, [%1];" : "=r"(v) : "r"(smem_u32addr(p)) : "memory");
-  return v;
+__device__ __forceinline__ void sts_addr(uint32_t addr, uint32_t v) {
+  asm volatile("st.shared.b32 [%0], %1;" ::"r"(addr), "r"(v) : "memory");
 }
-__device__ __forceinline__ uint64_t lds_key(const uint64_t* p) {
-  uint64_t v;
-  asm volatile("ld.shared.b64 %0, [%1];" : "=l"(v) : "r"(smem_u32addr(p)) : "memory");
-  return v;
+__device__ __forceinline__ void sts_addr(uint32_t addr, uint64_t v) {
+  asm volatile("st.shared.b64 [%0], %1;" ::"r"(addr), "l"(v) : "memory");
+}
+__device__ __forceinline__ void sts128(uint32_t addr, const uint32_t* v) {
+  asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(addr), "r"(v[0]), "r"(v[1]),
+               "r"(v[2]), "r"(v[3])
+               : "memory");
+}
+__device__ __forceinline__ void sts128(uint32_t addr, const uint64_t* v) {
+  asm volatile("st.shared.v2.b64 [%0], {%1, %2};" ::"r"(addr), "l"(v[0]), "l"(v[1]) : "memory");
+}
+
+template <typename KeyT>
+__device__ __forceinline__ KeyT lds_at(uint32_t addr) {
+  if constexpr (sizeof(KeyT) == 4) {
+    uint32_t v;
+    asm volatile("ld.shared.b32 %0, [%1];" : "=r"(v) : "r"(addr) : "memory");
+    return v;
+  } else {
+    uint64_t v;
+    asm volatile("ld.shared.b64 %0, [%1];" : "=l"(v) : "r"(addr) : "memory");
+    return v;
+  }
+}
+__device__ __forceinline__ void lds_chunk(uint32_t addr, uint32_t* v) {
+  asm volatile("ld.shared.v4.b32 {%0, %1, %2, %3}, [%4];"
+               : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3])
+               : "r"(addr)
+               : "memory");
+}
+__device__ __forceinline__ void lds_chunk(uint32_t addr, uint64_t* v) {
+  asm volatile("ld.shared.v2.b64 {%0, %1}, [%2];" : "=l"(v[0]), "=l"(v[1]) : "r"(addr) : "memory");
+}
+
+template <typename KeyT>
+__device__ __forceinline__ KeyT lds_key(const KeyT* p) {
+  return lds_at<KeyT>(smem_u32addr(p));
 }
 // v = a[0] when idx < lim (signed), b[0] otherwise: one compare, two predicated
 // loads with complementary predicates (each touching consecutive words only).
@@ -355,7 +386,7 @@ __device__ __forceinline__ int warp_corank(const KeyT* A, int lenA, const KeyT* 
 
 // Both co-ranks of a block, of d and of d + m, in one search: lanes 0-15 look
 // for the first, lanes 16-31 for the second, each 16 probes a round (an odd
-// stride: at most two probes per bank).  Up to 4912 items in three rounds; one after
+// stride: at most two probes per bank).  Up to 4368 items in three rounds; one after
 // the other, 32 probes each, took five dependent rounds (the second search
 // bracketed by the first).
 template <typename KeyT>
@@ -503,10 +534,6 @@ __device__ __forceinline__ uint4 lds128(uint32_t addr) {
                : "memory");
   return x;
 }
-__device__ __forceinline__ void sts32(uint32_t addr, uint32_t v) {
-  asm volatile("st.shared.b32 [%0], %1;" ::"r"(addr), "r"(v) : "memory");
-}
-
 // Rows 4q .. 4q + 3 of the striped layout to addr (+ 128: the high halves of 8-byte keys).
 __device__ __forceinline__ void store_rows4(uint32_t addr, const uint32_t* v) {
   stsm_x4(addr, v[0], v[1], v[2], v[3]);
@@ -516,10 +543,10 @@ __device__ __forceinline__ void store_rows4(uint32_t addr, const uint64_t* v) {
   stsm_x4(addr + 128, (uint32_t)(v[0] >> 32), (uint32_t)(v[1] >> 32), (uint32_t)(v[2] >> 32),
           (uint32_t)(v[3] >> 32));
 }
-__device__ __forceinline__ void store_word(uint32_t addr, uint32_t v) { sts32(addr, v); }
+__device__ __forceinline__ void store_word(uint32_t addr, uint32_t v) { sts_addr(addr, v); }
 __device__ __forceinline__ void store_word(uint32_t addr, uint64_t v) {
-  sts32(addr, (uint32_t)v);
-  sts32(addr + 128, (uint32_t)(v >> 32));
+  sts_addr(addr, (uint32_t)v);
+  sts_addr(addr + 128, (uint32_t)(v >> 32));
 }
 // Keys 4 ch .. 4 ch + 3 of a row from the chunk at addr (+ 128 as above).
 __device__ __forceinline__ void load_chunk(uint32_t addr, uint32_t* v) {
@@ -627,43 +654,6 @@ __device__ __forceinline__ void warp_bitonic_1024(KeyT (&v)[32], KeyT* out, int 
   striped_to_blocked(v, out, nr, lane);
   blocked_stages<FLIP>(v, lane, c);                  // strides 16 .. 1
 }
-__device__ __forceinline__ void sts_addr(uint32_t addr, uint32_t v) {
-  asm volatile("st.shared.b32 [%0], %1;" ::"r"(addr), "r"(v) : "memory");
-}
-__device__ __forceinline__ void sts_addr(uint32_t addr, uint64_t v) {
-  asm volatile("st.shared.b64 [%0], %1;" ::"r"(addr), "l"(v) : "memory");
-}
-__device__ __forceinline__ void sts128(uint32_t addr, const uint32_t* v) {
-  asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(addr), "r"(v[0]), "r"(v[1]),
-               "r"(v[2]), "r"(v[3])
-               : "memory");
-}
-__device__ __forceinline__ void sts128(uint32_t addr, const uint64_t* v) {
-  asm volatile("st.shared.v2.b64 [%0], {%1, %2};" ::"r"(addr), "l"(v[0]), "l"(v[1]) : "memory");
-}
-
-template <typename KeyT>
-__device__ __forceinline__ KeyT lds_at(uint32_t addr) {
-  if constexpr (sizeof(KeyT) == 4) {
-    uint32_t v;
-    asm volatile("ld.shared.b32 %0, [%1];" : "=r"(v) : "r"(addr) : "memory");
-    return v;
-  } else {
-    uint64_t v;
-    asm volatile("ld.shared.b64 %0, [%1];" : "=l"(v) : "r"(addr) : "memory");
-    return v;
-  }
-}
-__device__ __forceinline__ void lds_chunk(uint32_t addr, uint32_t* v) {
-  asm volatile("ld.shared.v4.b32 {%0, %1, %2, %3}, [%4];"
-               : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3])
-               : "r"(addr)
-               : "memory");
-}
-__device__ __forceinline__ void lds_chunk(uint32_t addr, uint64_t* v) {
-  asm volatile("ld.shared.v2.b64 {%0, %1}, [%2];" : "=l"(v[0]), "=l"(v[1]) : "r"(addr) : "memory");
-}
-
 // 16-byte store when a <= b (signed), compare and store in one predicate.
 __device__ __forceinline__ void sts128_if_le(uint32_t addr, const uint32_t* v, int a, int b) {
   asm volatile(

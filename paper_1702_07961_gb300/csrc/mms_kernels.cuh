@@ -60,7 +60,6 @@ inline bool valid_tile_warps(int key_bytes, int w) {
 }
 
 size_t tile_sort_smem_bytes(int key_bytes, int warps);
-size_t merge_pass_smem_bytes(int key_bytes, int warps, int K);
 
 // Base case: sorts every tile of 1024 * tile_warps keys; in == out allowed.
 // xin / xout: apply the float order transform on load / its inverse on store.

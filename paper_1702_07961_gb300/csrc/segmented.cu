@@ -441,7 +441,7 @@ int sm_count() {
 
 // Sets a kernel's dynamic shared-memory limit, except while `s` is being
 // captured into a graph: the capture is preceded by a preparing pass that
-// sets every attribute (attribute calls are not stream work).
+// sets it (attribute calls are not stream work).
 template <typename Kern>
 cudaError_t set_smem(Kern k, size_t bytes, cudaStream_t s) {
   cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
@@ -468,10 +468,9 @@ template <typename KeyT, int WARPS, bool XIN>
 cudaError_t launch_seg_tile(const void* keys_in, void* a, void* b, const Desc* desc,
                             const int* total, long long upper, cudaStream_t s) {
   auto k = seg_tile_sort_kernel<KeyT, WARPS, XIN>;
-  const size_t smem = tile_sort_smem_bytes(sizeof(KeyT), WARPS);
-  cudaError_t e = set_smem(k, smem, s);
+  const size_t smem = tile_sort_smem_bytes(sizeof(KeyT), WARPS);      // at most 48 KB: no attribute
   unsigned grid = 1;
-  if (e == cudaSuccess) e = persistent_grid(k, WARPS * 32, smem, upper, &grid);
+  const cudaError_t e = persistent_grid(k, WARPS * 32, smem, upper, &grid);
   if (e != cudaSuccess) return e;
   return launch_k(k, dim3(grid), dim3(WARPS * 32), smem, s, true, static_cast<const KeyT*>(keys_in),
                   static_cast<KeyT*>(a), static_cast<KeyT*>(b), desc, total, upper);
@@ -481,10 +480,9 @@ template <int WARPS, bool XIN>
 cudaError_t launch_seg_tile_comp(const void* keys_in, void* a, void* b, const Desc* desc,
                                  const int* total, long long upper, cudaStream_t s) {
   auto k = seg_tile_sort_composite_kernel<WARPS, XIN>;
-  const size_t smem = tile_sort_smem_bytes(8, WARPS);
-  cudaError_t e = set_smem(k, smem, s);
+  const size_t smem = tile_sort_smem_bytes(8, WARPS);      // at most 48 KB: no attribute
   unsigned grid = 1;
-  if (e == cudaSuccess) e = persistent_grid(k, WARPS * 32, smem, upper, &grid);
+  const cudaError_t e = persistent_grid(k, WARPS * 32, smem, upper, &grid);
   if (e != cudaSuccess) return e;
   // The value copy lies between this and the planner: the launch takes no early start then.
   return launch_k(k, dim3(grid), dim3(WARPS * 32), smem, s, true,
@@ -581,32 +579,16 @@ cudaError_t seg_round(int unit_bytes, int tw, bool is_f32, int kmax, bool small,
   return cudaErrorInvalidValue;
 }
 
-// Sets the shared-memory attribute of every kernel a batch of this shape
-// launches (before a graph capture, during which attributes are not set).
-mms_status seg_prepare(mms_key_type kt, bool pairs, int tw) {
-  cudaError_t e = cudaSuccess;
-  const bool f = kt == MMS_KEY_F32;
-  if (pairs) {
-    const size_t t = tile_sort_smem_bytes(8, tw);
-    if (tw == 4) e = f ? set_smem_limit(seg_tile_sort_composite_kernel<4, true>, t) : set_smem_limit(seg_tile_sort_composite_kernel<4, false>, t);
-    if (tw == 2) e = f ? set_smem_limit(seg_tile_sort_composite_kernel<2, true>, t) : set_smem_limit(seg_tile_sort_composite_kernel<2, false>, t);
-  } else if (kt == MMS_KEY_U64) {
-    const size_t t = tile_sort_smem_bytes(8, tw);
-    if (tw == 4) e = set_smem_limit(seg_tile_sort_kernel<uint64_t, 4, false>, t);
-    if (tw == 2) e = set_smem_limit(seg_tile_sort_kernel<uint64_t, 2, false>, t);
+// Sets the shared-memory limit of the merge kernel a batch of this shape launches
+// (before a graph capture, during which it is not set).
+mms_status seg_prepare(int unit_bytes, int tw) {
+  cudaError_t e = cudaErrorInvalidValue;
+  if (unit_bytes == 8) {
+    if (tw == 4) e = set_smem_limit(seg_merge_kernel<uint64_t, 4>, seg_merge_max_smem<uint64_t, 4>());
+    if (tw == 2) e = set_smem_limit(seg_merge_kernel<uint64_t, 2>, seg_merge_max_smem<uint64_t, 2>());
   } else {
-    const size_t t = tile_sort_smem_bytes(4, tw);
-    if (tw == 8) e = f ? set_smem_limit(seg_tile_sort_kernel<uint32_t, 8, true>, t) : set_smem_limit(seg_tile_sort_kernel<uint32_t, 8, false>, t);
-    if (tw == 4) e = f ? set_smem_limit(seg_tile_sort_kernel<uint32_t, 4, true>, t) : set_smem_limit(seg_tile_sort_kernel<uint32_t, 4, false>, t);
-  }
-  if (e == cudaSuccess) {
-    if (pairs || kt == MMS_KEY_U64) {
-      if (tw == 4) e = set_smem_limit(seg_merge_kernel<uint64_t, 4>, seg_merge_max_smem<uint64_t, 4>());
-      if (tw == 2) e = set_smem_limit(seg_merge_kernel<uint64_t, 2>, seg_merge_max_smem<uint64_t, 2>());
-    } else {
-      if (tw == 8) e = set_smem_limit(seg_merge_kernel<uint32_t, 8>, seg_merge_max_smem<uint32_t, 8>());
-      if (tw == 4) e = set_smem_limit(seg_merge_kernel<uint32_t, 4>, seg_merge_max_smem<uint32_t, 4>());
-    }
+    if (tw == 8) e = set_smem_limit(seg_merge_kernel<uint32_t, 8>, seg_merge_max_smem<uint32_t, 8>());
+    if (tw == 4) e = set_smem_limit(seg_merge_kernel<uint32_t, 4>, seg_merge_max_smem<uint32_t, 4>());
   }
   return e == cudaSuccess ? MMS_OK : seg_fail(MMS_ERR_CUDA, cudaGetErrorString(e));
 }
@@ -727,7 +709,7 @@ static mms_status seg_sort_impl(mms_key_type kt, void* d_keys, uint32_t* d_value
   for (int c = 0; c <= size_class(mx); ++c) kmax = P.class_fanout[c] > kmax ? P.class_fanout[c] : kmax;
   P.kmax = kmax;
 
-  if (prepare_only) return seg_prepare(kt, pairs, tw);
+  if (prepare_only) return seg_prepare(unit, tw);
 
   int ev = 0;
   auto mark = [&]() {

@@ -143,10 +143,7 @@ __device__ __forceinline__ Item<KeyT> shfl_item(unsigned gm, const Item<KeyT>& i
 // are the lane's run and its length (rlen = 0 when !act); the runs may lie in
 // global or in shared memory.  Arguments other than run / rlen / act are
 // uniform over the lane group; every lane of it must call.
-// UNSWITCH: one drop loop per arg-max form (no pad test inside the loop);
-// measured faster in the splitter kernel (splitter_row), slower inside the
-// much larger partition merge kernel, which takes the default single loop.
-template <typename KeyT, typename Idx, bool UNSWITCH = false>
+template <typename KeyT, typename Idx>
 __device__ __forceinline__ Idx multiseq_pivot(const KeyT* run, Idx rlen, bool act, int K, Idx k,
                                               unsigned gm) {
   const int lane = threadIdx.x & 31;
@@ -221,17 +218,9 @@ __device__ __forceinline__ Idx multiseq_pivot(const KeyT* run, Idx rlen, bool ac
         }
       }
     };
-    if constexpr (UNSWITCH) {
-      if (any_pad) {
-        for (Idx p = 0; p < pops; ++p) drop(grp_argmax(gm, act && cnt >= 1, top));
-      } else {
-        for (Idx p = 0; p < pops; ++p) drop(grp_argmax_real(gm, act && cnt >= 1, top.key));
-      }
-    } else {
-      for (Idx p = 0; p < pops; ++p)
-        drop(any_pad ? grp_argmax(gm, act && cnt >= 1, top)
-                     : grp_argmax_real(gm, act && cnt >= 1, top.key));
-    }
+    for (Idx p = 0; p < pops; ++p)
+      drop(any_pad ? grp_argmax(gm, act && cnt >= 1, top)
+                   : grp_argmax_real(gm, act && cnt >= 1, top.key));
     d = cnt;
     e = top;
     pad_prev = any_pad;

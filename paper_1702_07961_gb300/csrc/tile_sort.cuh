@@ -116,12 +116,6 @@ __device__ __forceinline__ KeyT xform_in(KeyT k) {
   if constexpr (XIN) return (KeyT)f32_to_ordered((uint32_t)k);
   return k;
 }
-template <typename KeyT, bool XOUT>
-__device__ __forceinline__ KeyT xform_out(KeyT k) {
-  if constexpr (XOUT) return (KeyT)ordered_to_f32((uint32_t)k);
-  return k;
-}
-
 // Writes the sorted tile src[0, m) to global memory: one TMA bulk store of the
 // 16-byte-aligned body, plain stores for the < 16-byte tail.  Every thread
 // must call it (it contains a barrier).
