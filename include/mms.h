@@ -112,8 +112,12 @@ size_t mms_sort_workspace_bytes(mms_key_type kt, size_t n, int with_values);
  * contents: its status word is cleared on `stream` first), or NULL to let the
  * library allocate one stream-ordered (cudaMallocAsync) and free it after the
  * sort; the call then still returns without waiting for the GPU, and its
- * device-side status goes to the word mms_stream_status() reads.  n = 0 and
- * n = 1 are no-ops. */
+ * device-side status goes to the word mms_stream_status() reads.  That memory
+ * comes from the device's default pool.  Unless the program has raised the
+ * pool's release threshold, every synchronisation gives it back, and a sort
+ * right after one pays for mapping it again (2^20 keys and a wait: 247 us
+ * against 64 with a workspace of the caller's), so a program that waits for
+ * its sorts one by one had better pass its own.  n = 0 and n = 1 are no-ops. */
 mms_status mms_sort_keys(mms_key_type kt, void* d_keys, size_t n, void* d_ws, size_t ws_bytes,
                          void* stream);
 mms_status mms_sort_keys_ex(mms_key_type kt, void* d_keys, size_t n, void* d_ws, size_t ws_bytes,
@@ -222,8 +226,9 @@ mms_status mms_merge_pass_pipelined(mms_key_type kt, const void* d_in, void* d_o
  * segment gets the fanout K of its size class ceil(log2 n) and its own number
  * of rounds; the whole launch sequence needs no host synchronisation, so it
  * can be captured into a CUDA graph (mms_segmented_graph_create).  Offsets
- * out of order, or a segment above max_segment_items, set the workspace
- * status word to MMS_ERR_INTERNAL (read it with mms_workspace_status). */
+ * out of order, or a segment above max_segment_items that needs more merge
+ * rounds than that maximum does, set the workspace status word to
+ * MMS_ERR_INTERNAL (read it with mms_workspace_status). */
 typedef struct {
   int class_fanout[33];       /* K (2..32) for segments of size class c = ceil(log2 n); 0 =
                                  default (4 for 4-byte keys, 8 for 8-byte keys and key-value

@@ -1,14 +1,15 @@
 // splitter.cuh -- parallel partitioning of a K-way merge round (Sec. 4.1),
 // shared by the whole-array splitter and the segmented (batched) one.
 //
-// For every output tile j of every group of K sorted runs, one lane group
-// (W >= K lanes, 32 / W groups per warp) finds the pivot indices c[r]
-// (r < K): the number of items run r contributes to the group's first j*S
+// For every output tile j of every group of K sorted runs, one warp finds the pivot indices
+// c[r] (r < K): the number of items run r contributes to the group's first j*S
 // outputs under the strict order (key, run, position).  That
 // order makes the pivots unique even with repeated keys (the paper's
 // non-overlap condition, read on the composite key) and equals a stable merge.
 //
-// Search (one lane per run, K <= 32): stride halving on regular samples.  At
+// Two searches.  window_pivot is the splitter kernels': windows of samples, sorted across
+// the warp (described there).  multiseq_pivot, one lane per run (K <= 32), is the
+// partition variant's, on segments in shared memory: stride halving on regular samples.  At
 // stride s the lane group holds the exact pivots d of the s-sample problem -- the
 // items at positions s-1, 2s-1, ... of every run -- for rank floor(k/s).
 // Halving s adds one candidate per run just above its pivot; the pivots of the
@@ -137,7 +138,7 @@ __device__ __forceinline__ Item<KeyT> shfl_item(unsigned gm, const Item<KeyT>& i
   return o;
 }
 
-// The search itself: the lanes of the group (lane gb + r on run r, act for
+// Stride halving: the lanes of the group (lane gb + r on run r, act for
 // r < K) return the number of items each run contributes to the first k of
 // the K runs' merge under the order (key, run, position).  `run` and `rlen`
 // are the lane's run and its length (rlen = 0 when !act); the runs may lie in

@@ -26,7 +26,7 @@ namespace mms {
 // x = j + i with j running from k mod p in steps of 2k and i from 0 to k - 1,
 // whenever both lie in the same block of 2p items.  Every index is a
 // compile-time constant once the loops are unrolled, so each compare-exchange
-// is register to register; within a stage about two of three pairs take the
+// is register to register; within a stage the mix's share of the pairs takes the
 // multiply-add form (by their ordinal in the stage), as in the other networks.
 template <typename KeyT, typename M>
 __device__ __forceinline__ void lane_sort32(KeyT (&v)[32], const M& c) {
