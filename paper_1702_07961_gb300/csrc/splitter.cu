@@ -16,11 +16,19 @@ constexpr int kSplitterWarps = 4;
 // without, 66 with).
 constexpr long long kSplitterPdlTiles = 192;
 
+// Rows from which 8-byte keys with more than 4 runs take stride halving (K2 = 0).  Up to
+// about one wave of warps a row's chain of steps counts, and windows take a third of the steps;
+// beyond it the sectors, and 32 M samples of 8 bytes a step are twice a halving level's
+// share.  Sorts of u64 keys, us, windows / halving, random and 1% swapped keys: 6 * 10^6 (1465 rows) 355 / 379, 357 / 365;
+// 1.2 * 10^7 (2930) 709 / 721, 664 / 643; 1.6 * 10^7 (3907) 910 / 909, 863 / 807; 10^8 6338 / 6309, 5431 / 4967.
+// 4-byte keys stay with windows: 10^8 random u32 keys' splitters 264 / 307.
+constexpr unsigned kHalvingRows = 3584;
+
 // CTAs per SM the splitter is compiled for: 40 warps (48 registers), 32 with more than 16
 // runs, whose window is twice as large.  The search waits for loads, so warps count: left
 // to itself the compiler takes 40 to 64 and spills some (6 * 10^6 pairs of 4-byte keys 411 -> 414
 // us, 10^8 u32 keys' splitters 262 -> 266); for 48 warps it spills more (268).
-constexpr int splitter_ctas(int k2) { return k2 == 32 ? 8 : 10; }
+constexpr int splitter_ctas(int k2) { return k2 == 32 ? 8 : 10; }   // 48 registers halving, too
 
 template <typename KeyT, int K2, typename Idx>
 __global__ void __launch_bounds__(32 * kSplitterWarps, splitter_ctas(K2))
@@ -39,16 +47,22 @@ static cudaError_t launch_k2(const void* in, long long n, long long run_len, int
                              bool pdl) {
   const unsigned grid = (ntiles + kSplitterWarps - 1) / kSplitterWarps;
   const KeyT* kin = static_cast<const KeyT*>(in);
-  if (n < (1ll << 31))                            // counts and positions fit 32 bits
+  if (n < (K2 == 0 ? 1ll << 30 : 1ll << 31))      // counts and positions fit 32 bits
     return launch_k(splitter_kernel<KeyT, K2, int>, dim3(grid), dim3(32 * kSplitterWarps), 0, s, pdl, kin, n, run_len,
                     K, S, tpg, ntiles, table);
-  return launch_k(splitter_kernel<KeyT, K2, long long>, dim3(grid), dim3(32 * kSplitterWarps), 0, s, pdl, kin, n,
-                  run_len, K, S, tpg, ntiles, table);
+  if constexpr (sizeof(KeyT) == 8 && K2 > 4)
+    return cudaErrorInvalidValue;                 // so many rows have taken K2 = 0
+  else
+    return launch_k(splitter_kernel<KeyT, K2, long long>, dim3(grid), dim3(32 * kSplitterWarps), 0, s, pdl, kin, n,
+                    run_len, K, S, tpg, ntiles, table);
 }
 
 template <typename KeyT>
 static cudaError_t launch_key(const void* in, long long n, long long run_len, int K, long long S,
                               unsigned tpg, unsigned ntiles, long long* table, cudaStream_t s, bool pdl) {
+  if constexpr (sizeof(KeyT) == 8)
+    if (K > 4 && ntiles >= kHalvingRows)
+      return launch_k2<KeyT, 0>(in, n, run_len, K, S, tpg, ntiles, table, s, pdl);
   switch (pow2_ceil(K)) {
     case 2: return launch_k2<KeyT, 2>(in, n, run_len, K, S, tpg, ntiles, table, s, pdl);
     case 4: return launch_k2<KeyT, 4>(in, n, run_len, K, S, tpg, ntiles, table, s, pdl);

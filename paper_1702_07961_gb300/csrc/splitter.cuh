@@ -7,9 +7,9 @@
 // order makes the pivots unique even with repeated keys (the paper's
 // non-overlap condition, read on the composite key) and equals a stable merge.
 //
-// Two searches.  window_pivot is the splitter kernels': windows of samples, sorted across
-// the warp (described there).  multiseq_pivot, one lane per run (K <= 32), is the
-// partition variant's, on segments in shared memory: stride halving on regular samples.  At
+// Two searches.  window_pivot: windows of samples, sorted across the warp (described there).
+// multiseq_pivot, one lane per run (K <= 32), for large sorts of 8-byte keys and, on
+// segments in shared memory, for the partition variant: stride halving on regular samples.  At
 // stride s the lane group holds the exact pivots d of the s-sample problem -- the
 // items at positions s-1, 2s-1, ... of every run -- for rank floor(k/s).
 // Halving s adds one candidate per run just above its pivot; the pivots of the
@@ -144,7 +144,10 @@ __device__ __forceinline__ Item<KeyT> shfl_item(unsigned gm, const Item<KeyT>& i
 // are the lane's run and its length (rlen = 0 when !act); the runs may lie in
 // global or in shared memory.  Arguments other than run / rlen / act are
 // uniform over the lane group; every lane of it must call.
-template <typename KeyT, typename Idx>
+// UNSWITCH: one drop loop per arg-max form (no pad test inside the loop): in the splitter
+// kernel 10^8 u64 keys sort in 6309 us with it, 6321 without; in the much larger partition
+// merge kernel it is slower.
+template <typename KeyT, typename Idx, bool UNSWITCH = false>
 __device__ __forceinline__ Idx multiseq_pivot(const KeyT* run, Idx rlen, bool act, int K, Idx k,
                                               unsigned gm) {
   const int lane = threadIdx.x & 31;
@@ -219,9 +222,17 @@ __device__ __forceinline__ Idx multiseq_pivot(const KeyT* run, Idx rlen, bool ac
         }
       }
     };
-    for (Idx p = 0; p < pops; ++p)
-      drop(any_pad ? grp_argmax(gm, act && cnt >= 1, top)
-                   : grp_argmax_real(gm, act && cnt >= 1, top.key));
+    if constexpr (UNSWITCH) {
+      if (any_pad) {
+        for (Idx p = 0; p < pops; ++p) drop(grp_argmax(gm, act && cnt >= 1, top));
+      } else {
+        for (Idx p = 0; p < pops; ++p) drop(grp_argmax_real(gm, act && cnt >= 1, top.key));
+      }
+    } else {
+      for (Idx p = 0; p < pops; ++p)
+        drop(any_pad ? grp_argmax(gm, act && cnt >= 1, top)
+                     : grp_argmax_real(gm, act && cnt >= 1, top.key));
+    }
     d = cnt;
     e = top;
     pad_prev = any_pad;
@@ -229,7 +240,7 @@ __device__ __forceinline__ Idx multiseq_pivot(const KeyT* run, Idx rlen, bool ac
   return d;
 }
 
-// The search of the splitter kernels: the same pivots by the same idea --
+// The splitter kernels' search by windows: the same pivots by the same idea --
 // exact pivots of the s-sample problem, s shrinking to 1 -- but with a window
 // of W samples of every run held across the warp, so that a step divides s by
 // W / 2 instead of 2 and its drops are found together, not one arg-max at a
@@ -270,7 +281,7 @@ __device__ __forceinline__ Idx multiseq_pivot(const KeyT* run, Idx rlen, bool ac
 // about as long; above that the 32 M sectors a step reads.  Against stride halving (log2(K *
 // run_len) levels, each a load and about K / 2 arg-maxes of 250 cycles) on random keys: both
 // splitters of 2^20 u32 keys 41 -> 25 us, the three of 16.8 * 10^6 85 -> 59 us, the four of
-// 3 * 10^8 926 -> 811 us, the five of 10^8 u64 567 -> 596 us.  Finding the threshold by
+// 3 * 10^8 926 -> 811 us; with 8-byte keys large sorts keep stride halving (splitter.cu).  Finding the threshold by
 // quickselect instead of sorting took 500 cycles a round of 5 to 7 rounds and was no faster
 // than stride halving.
 
@@ -470,12 +481,14 @@ __device__ __forceinline__ Idx window_pivot(const KeyT* run, Idx rlen, Idx maxle
 // Pivots of output tile j of group g, found by one warp: row[r] receives the
 // number of items of run r among the group's first j * S outputs.  Arguments
 // are uniform over the warp.  Idx is the type of the counts and positions of
-// the search: int when n < 2^31, long long otherwise.  K2: K rounded up to a power of two.
+// the search: int when n < 2^31, long long otherwise.  K2: K rounded up to a power of two;
+// 0: the search by stride halving, with any K <= 32, whose positions take int when n < 2^30
+// only (every position probed stays below 2n).
 template <typename KeyT, int K2, typename Idx = long long>
 __device__ __forceinline__ void splitter_row(const KeyT* in, long long n,
                                              long long run_len, int K, long long S, long long g,
                                              long long j, long long* row) {
-  constexpr int SUB = 32 / K2;
+  constexpr int SUB = K2 == 0 ? 1 : 32 / (K2 == 0 ? 1 : K2);
   const int lane = threadIdx.x & 31;
   const int rr = lane / SUB;                    // run of this lane
   const bool act = rr < K;
@@ -484,7 +497,11 @@ __device__ __forceinline__ void splitter_row(const KeyT* in, long long n,
   rlen64 = rlen64 < 0 ? 0 : (rlen64 > run_len ? run_len : rlen64);
   const Idx rlen = act ? (Idx)rlen64 : Idx(0);
   const KeyT* run = in + (act ? rstart : 0);
-  const Idx d = window_pivot<KeyT, K2, Idx>(run, rlen, (Idx)(run_len < n ? run_len : n), (Idx)(j * S));
+  Idx d;
+  if constexpr (K2 == 0)
+    d = multiseq_pivot<KeyT, Idx, true>(run, rlen, act, K, (Idx)(j * S), 0xffffffffu);
+  else
+    d = window_pivot<KeyT, K2, Idx>(run, rlen, (Idx)(run_len < n ? run_len : n), (Idx)(j * S));
   if (act && lane % SUB == 0) row[rr] = d;
 }
 
