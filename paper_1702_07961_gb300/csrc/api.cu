@@ -121,8 +121,8 @@ bool valid_base_items(int key_bytes, int tw, int base_items) {
 // and then the rounds (e.g. (16,16,16,4) for 10^8 4-byte keys).  The choice is
 // a coin-change dynamic program over log2 of the coverage.  opt->fanout fixes
 // every round's K instead; the result does not depend on the plan.
-// Fitted before the splitter's last change; the fit since (0.190, 0.303, 0.433, 0.555, 0.794
-// and 0.416, 0.647, 0.947, 1.383, 2.354) changes no plan up to 2^32 items.
+// Fitted before the splitter's last changes; the fit since (0.189, 0.303, 0.433, 0.556, 0.794
+// and 0.414, 0.646, 0.940, 1.381, 2.293) changes no plan up to 2^32 items.
 namespace plan_model {
 // ms per 10^8 items of one round (merge pass + splitter), for K = 2, 4, 8, 16, 32
 constexpr double kCost4[5] = {0.194, 0.312, 0.444, 0.567, 0.805};   // 4-byte keys
